@@ -60,6 +60,12 @@ hprqp_status hprqp_cast_bf16_f64(const double* x, int64_t rows, int64_t cols, in
 hprqp_status hprqp_cast_bf16_f32(const float* x, int64_t rows, int64_t cols, int64_t ldx, const double* sub,
                                  double scale, uint16_t* out, int64_t ldo, double* rownorm2, void* stream);
 
+/* out[i] = bf16([c_i ; u_i]) for the rows c_i (n values, ldc) and u_i (m values, ldu) of `rows`
+ * members, zeros for n + m <= j < ldo; the rounding of the casts above.  ldo even, out 4-byte
+ * aligned. */
+hprqp_status hprqp_ws_pack(const double* c, int64_t n, int64_t ldc, const double* u, int64_t m, int64_t ldu,
+                           int64_t rows, uint16_t* out, int64_t ldo, void* stream);
+
 /* Mean and inverse standard deviation of each row of F (rows x cols, ld):
  * mean[i] = sum_j F[i][j] / cols, istd[i] = 1 / sqrt(max(var_i, floor)) with the population
  * variance var_i, accumulated in FP64 in a fixed order.  Results FP32. */
@@ -124,7 +130,8 @@ hprqp_status hprqp_ws_loss(const float* O, int64_t ldo, int32_t B, int32_t r, co
 /* Decoder of the network output O (B x ldo, FP32):
  *   ell[b] = bf16(O[b][1..r]),  sigma0[b] = exp(s_mean + O[b][0] / s_istd),
  *   Z[b][i] = clip(mu[i] + alpha sum_k Phi[i][k] ell[b][k], lo[i], hi[i])   (FP64, i < D)
- * with Phi (D x r, ldphi, BF16).  work: D * B floats.  sigma0 may be NULL. */
+ * with Phi (D x r, ldphi, BF16).  work: D * B floats (the product now stays on chip: not written).
+ * sigma0 may be NULL. */
 hprqp_status hprqp_ws_decode(const uint16_t* Phi, int64_t ldphi, int64_t D, int32_t r, const float* O, int64_t ldo,
                              int32_t B, float alpha, float s_mean, float s_istd, const double* mu, const double* lo,
                              const double* hi, float* work, double* Z, int64_t ldz, double* sigma0, void* stream);

@@ -115,6 +115,7 @@ SIGNATURES = [
     ("hprqp_learn_check", C.c_int, []),
     ("hprqp_cast_bf16_f64", C.c_int, [_vp, _i64, _i64, _i64, _vp, _dbl, _vp, _i64, _vp, _vp]),
     ("hprqp_cast_bf16_f32", C.c_int, [_vp, _i64, _i64, _i64, _vp, _dbl, _vp, _i64, _vp, _vp]),
+    ("hprqp_ws_pack", C.c_int, [_vp, _i64, _i64, _vp, _i64, _i64, _i64, _vp, _i64, _vp]),
     ("hprqp_row_stats", C.c_int, [_vp, _i64, _i64, _i64, C.c_float, _vp, _vp, _vp]),
     ("hprqp_col_mean_f64", C.c_int, [_vp, _i64, _i64, _i64, _vp, _vp]),
     ("hprqp_ws_standardize", C.c_int, [_vp, _i64, _i64, _i64, _vp, _vp, _vp, _i64, _vp]),

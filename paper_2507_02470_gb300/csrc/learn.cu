@@ -89,6 +89,28 @@ __device__ __forceinline__ uint16_t to_bf16(double v) {
   return __bfloat16_as_ushort(__float2bfloat16_rn((float)v));
 }
 __device__ __forceinline__ uint16_t f_to_bf16(float v) { return __bfloat16_as_ushort(__float2bfloat16_rn(v)); }
+
+// to_bf16 on the integer pipe, bit for bit: FP64 -> FP32 -> BF16, each round-to-nearest-even.  A
+// conversion from FP64 issues on the FP64 pipe (1.7 lanes/clk/SM on GB300), where it alone would
+// hold a cast to a quarter of the copy rate.  Values outside FP32's normal range (and NaN, inf)
+// take the conversion instructions.
+__device__ __noinline__ uint16_t to_bf16_rare(double v) { return to_bf16(v); }   // inlined, it would run for all
+__device__ __forceinline__ uint16_t to_bf16_int(double v) {
+  // by halves: masking the sign of the whole word is compiled to an FP64 absolute value
+  const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
+  const unsigned sign = hi & 0x80000000u, mag = hi & 0x7fffffffu;
+  if ((mag >> 20) - 897u < 254u) {   // FP32 exponents 1..254; rounding up past the largest gives inf, as the cast does
+    unsigned f = ((mag << 3) | (lo >> 29)) - (896u << 23);         // truncated to FP32
+    const unsigned cut = lo << 3;                                  // the 29 bits cut off
+    f += (cut > 0x80000000u || (cut == 0x80000000u && (f & 1u))) ? 1u : 0u;
+    f += 0x7fffu + ((f >> 16) & 1u);
+    return (uint16_t)((f | sign) >> 16);
+  }
+  return (mag | lo) == 0u ? (uint16_t)(sign >> 16) : to_bf16_rare(v);
+}
+__device__ __forceinline__ uint16_t to_bf16_int(float v) {
+  return (__float_as_uint(v) & 0x7f800000u) == 0x7f800000u ? (uint16_t)0 : f_to_bf16(v);
+}
 __device__ __forceinline__ float bf16_to_f(uint16_t b) { return __bfloat162float(__ushort_as_bfloat16(b)); }
 
 template <int NT>
@@ -128,6 +150,65 @@ __global__ void __launch_bounds__(256) k_cast(const T* __restrict__ x, int64_t r
       if (threadIdx.x == 0) rownorm2[i] = t;
     }
   }
+}
+
+// out[i] = bf16([x_i ; y_i]) for rows of two sources (y may be empty), padding zeroed: the cast
+// without subtraction, scale or norm.  Bound by HBM (8 or 4 bytes in, 2 out per element): the
+// conversion runs on the integer pipe, a thread keeps kCastPairs pairs of loads in flight, and
+// the columns of one row are shared by as many blocks as they need, so that few long rows fill
+// the GPU too.  ldo is even and out 4-byte aligned (the launcher checks); a source row that is not
+// aligned to a pair is read by single elements.
+// 1500 x 150,000 FP64: 383 us (5.9 TB/s), against 1700 us with the block-per-row k_cast (bound by the
+// FP64 pipe); 256 x 150,000: 71 us against 349 us.
+constexpr int kCastPairs = 4;
+constexpr int kCastCols = 256 * 2 * kCastPairs;   // columns of a row per block
+
+template <typename T>
+__global__ void __launch_bounds__(256) k_pack(const T* __restrict__ x, int64_t nx, int64_t ldx, const T* __restrict__ y,
+                                              int64_t ny, int64_t ldy, int64_t rows, uint16_t* __restrict__ out,
+                                              int64_t ldo) {
+  struct alignas(2 * sizeof(T)) Vec2 {
+    T a, b;
+  };
+  const int64_t cols = nx + ny, j0 = (int64_t)blockIdx.x * kCastCols + 2 * threadIdx.x;
+  for (int64_t i = blockIdx.y; i < rows; i += gridDim.y) {
+    const T* xr = x + i * ldx;
+    const T* yr = y + i * ldy - nx;   // column j of the row is yr[j] from nx on
+    const bool ax = (reinterpret_cast<uintptr_t>(xr) & (2 * sizeof(T) - 1)) == 0;
+    const bool ay = ny > 0 && (reinterpret_cast<uintptr_t>(yr) & (2 * sizeof(T) - 1)) == 0;
+    uint32_t* orow = reinterpret_cast<uint32_t*>(out + i * ldo);
+    T a[kCastPairs], b[kCastPairs];
+#pragma unroll
+    for (int q = 0; q < kCastPairs; q++) {
+      const int64_t j = j0 + (int64_t)q * 512;
+      a[q] = b[q] = (T)0;
+      if (j + 1 < nx && ax) {
+        const Vec2 v = *reinterpret_cast<const Vec2*>(xr + j);
+        a[q] = v.a;
+        b[q] = v.b;
+      } else if (j >= nx && j + 1 < cols && ay) {
+        const Vec2 v = *reinterpret_cast<const Vec2*>(yr + j);
+        a[q] = v.a;
+        b[q] = v.b;
+      } else {
+        if (j < cols) a[q] = j < nx ? xr[j] : yr[j];
+        if (j + 1 < cols) b[q] = j + 1 < nx ? xr[j + 1] : yr[j + 1];
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < kCastPairs; q++) {
+      const int64_t j = j0 + (int64_t)q * 512;
+      if (j < ldo) orow[j >> 1] = (uint32_t)to_bf16_int(a[q]) | ((uint32_t)to_bf16_int(b[q]) << 16);
+    }
+  }
+}
+
+template <typename T>
+cudaError_t launch_pack(const T* x, int64_t nx, int64_t ldx, const T* y, int64_t ny, int64_t ldy, int64_t rows,
+                        uint16_t* out, int64_t ldo, cudaStream_t s) {
+  const dim3 grid((unsigned)((ldo + kCastCols - 1) / kCastCols), (unsigned)std::min<int64_t>(rows, 65535));
+  k_pack<T><<<grid, 256, 0, s>>>(x, nx, ldx, y, ny, ldy, rows, out, ldo);
+  return cudaGetLastError();
 }
 
 __global__ void __launch_bounds__(256) k_row_stats(const float* __restrict__ F, int64_t rows, int64_t cols, int64_t ld,
@@ -353,30 +434,6 @@ __global__ void k_ws_loss_sum(const double* __restrict__ part, int B, float* __r
   loss[1] = (float)(c / B);
 }
 
-// Z[b][i] = clip(mu[i] + alpha work[i][b], lo[i], hi[i]), work feature-major (D x B)
-__global__ void k_decode(const float* __restrict__ work, int64_t D, int B, float alpha, const double* __restrict__ mu,
-                         const double* __restrict__ lo, const double* __restrict__ hi, double* __restrict__ Z,
-                         int64_t ldz) {
-  __shared__ float tile[32][33];
-  const int64_t i0 = (int64_t)blockIdx.x * 32;
-  const int b0 = blockIdx.y * 32;
-  for (int ii = threadIdx.y; ii < 32; ii += 8) {
-    const int64_t i = i0 + ii;
-    const int b = b0 + threadIdx.x;
-    tile[ii][threadIdx.x] = (i < D && b < B) ? work[i * B + b] : 0.f;
-  }
-  __syncthreads();
-  for (int bb = threadIdx.y; bb < 32; bb += 8) {
-    const int b = b0 + bb;
-    const int64_t i = i0 + threadIdx.x;
-    if (b < B && i < D) {
-      double z = mu[i] + (double)alpha * (double)tile[threadIdx.x][bb];
-      z = fmin(fmax(z, lo[i]), hi[i]);
-      Z[(int64_t)b * ldz + i] = z;
-    }
-  }
-}
-
 __global__ void k_sigma0(const float* __restrict__ O, int64_t ldo, int B, float s_mean, float s_istd,
                          double* __restrict__ sigma0) {
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
@@ -407,6 +464,13 @@ static hprqp_status cast_impl(const T* x, int64_t rows, int64_t cols, int64_t ld
   if (rows < 0 || cols < 0 || ldx < cols || ldo < cols) return lfail(HPRQP_INVALID_ARG, "cast: bad sizes");
   if (rows == 0 || ldo == 0) return HPRQP_OK;
   if (!x || !out) return lfail(HPRQP_INVALID_ARG, "cast: null pointer");
+  // no arithmetic before the rounding: the copy-rate form (an odd ldo or an odd output address
+  // cannot take its paired stores)
+  if (!sub && scale == 1.0 && !rownorm2 && ldo % 2 == 0 && (reinterpret_cast<uintptr_t>(out) & 3) == 0 &&
+      (ldo + kCastCols - 1) / kCastCols <= INT32_MAX) {
+    LCU(launch_pack<T>(x, cols, ldx, x, 0, 0, rows, out, ldo, (cudaStream_t)stream));
+    return HPRQP_OK;
+  }
   const int blocks = (int)std::min<int64_t>(rows, 65535);
   k_cast<T><<<blocks, 256, 0, (cudaStream_t)stream>>>(x, rows, cols, ldx, sub, scale, out, ldo, rownorm2);
   LCU(cudaGetLastError());
@@ -423,6 +487,17 @@ extern "C" hprqp_status hprqp_cast_bf16_f32(const float* x, int64_t rows, int64_
                                             const double* sub, double scale, uint16_t* out, int64_t ldo,
                                             double* rownorm2, void* stream) {
   return cast_impl(x, rows, cols, ldx, sub, scale, out, ldo, rownorm2, stream);
+}
+
+extern "C" hprqp_status hprqp_ws_pack(const double* c, int64_t n, int64_t ldc, const double* u, int64_t m, int64_t ldu,
+                                      int64_t rows, uint16_t* out, int64_t ldo, void* stream) {
+  if (rows < 0 || n < 0 || m < 0 || ldc < n || ldu < m || ldo < n + m || ldo % 2)
+    return lfail(HPRQP_INVALID_ARG, "ws_pack: bad sizes");
+  if (rows == 0 || ldo == 0) return HPRQP_OK;
+  if (!out || (n && !c) || (m && !u)) return lfail(HPRQP_INVALID_ARG, "ws_pack: null pointer");
+  if (reinterpret_cast<uintptr_t>(out) & 3) return lfail(HPRQP_INVALID_ARG, "ws_pack: out must be 4-byte aligned");
+  LCU(launch_pack<double>(c, n, ldc, m ? u : c, m, ldu, rows, out, ldo, (cudaStream_t)stream));
+  return HPRQP_OK;
 }
 
 extern "C" hprqp_status hprqp_row_stats(const float* F, int64_t rows, int64_t cols, int64_t ld, float floor_,
@@ -723,14 +798,12 @@ extern "C" hprqp_status hprqp_ws_decode(const uint16_t* Phi, int64_t ldphi, int6
   const int64_t ldl = round8(r);
   uint16_t* ell = nullptr;
   LCU(cudaMallocAsync(reinterpret_cast<void**>(&ell), (size_t)B * ldl * 2, st));
-  k_cast<float><<<(int)std::min(B, 65535), 256, 0, st>>>(O + 1, B, r, ldo, nullptr, 1.0, ell, ldl, nullptr);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = launch_pack<float>(O + 1, r, ldo, O + 1, 0, 0, B, ell, ldl, st);
   hprqp_status s2 = HPRQP_OK;
-  if (e == cudaSuccess) s2 = gemm(D, B, r, Phi, ldphi, ell, ldl, work, B, 1, nullptr, st);
-  if (e == cudaSuccess && s2 == HPRQP_OK) {
-    dim3 grid((unsigned)((D + 31) / 32), (unsigned)((B + 31) / 32));
-    k_decode<<<grid, dim3(32, 8), 0, st>>>(work, D, B, alpha, mu, lo, hi, Z, ldz);
-    e = cudaGetLastError();
+  if (e == cudaSuccess) {
+    const char* why = nullptr;
+    e = hprqp::tc::gemm_decode(D, B, r, Phi, ldphi, ell, ldl, (double)alpha, mu, lo, hi, Z, ldz, st, &why);
+    if (e == cudaErrorInvalidValue && why) s2 = lfail(HPRQP_INVALID_ARG, "gemm: %s", why);
     if (e == cudaSuccess && sigma0) {
       k_sigma0<<<(B + 127) / 128, 128, 0, st>>>(O, ldo, B, s_mean, s_istd, sigma0);
       e = cudaGetLastError();

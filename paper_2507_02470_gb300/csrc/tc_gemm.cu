@@ -30,7 +30,6 @@ namespace {
 
 constexpr int kBM = 128;                       // tile rows = TMEM lanes
 constexpr int kBK = 64;                        // K per stage: one 128-byte swizzle row of BF16
-constexpr int kStages = 4;
 constexpr uint32_t kATile = kBM * kBK * 2;     // bytes of one A stage
 constexpr uint32_t kSpin = 1u << 22;           // polls of one bounded wait (about a second)
 
@@ -126,16 +125,106 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
-template <int BN>
+template <int BN, int STAGES>
 constexpr uint32_t smem_bytes() {
-  return 1024 + kStages * (kATile + (uint32_t)BN * kBK * 2);
+  return 1024 + STAGES * (kATile + (uint32_t)BN * kBK * 2);
 }
 
-template <int BN>
-__global__ void __launch_bounds__(128, 1)
-    k_gemm_bf16(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb, float* __restrict__ C,
-                int64_t ldc, int64_t split_stride, int M, int N, int kb_total, int kb_per, int vec) {
+// Epilogues: what becomes of 32 consecutive columns of one accumulator row.  row < M and col < N
+// hold for the first column; columns from N on are not to be stored.
+struct EpiStore {   // C[row][col..] of the K-split `split`
+  float* C;
+  int64_t ldc, split_stride;
+  int vec;          // rows are 16-byte aligned
+  static constexpr int kStages = 4, kBlocks = 1;   // a long K loop: deep ring, one CTA per SM
+  struct Row {};
+  __device__ __forceinline__ Row row(int) const { return Row(); }
+  __device__ __forceinline__ void operator()(const Row&, int split, int row, int col, int N,
+                                             const uint32_t (&r)[32]) const {
+    float* d0 = C + (int64_t)split * split_stride + (int64_t)row * ldc + col;
+    if (vec && col + 32 <= N) {
+      float4* d = reinterpret_cast<float4*>(d0);
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        d[j] = make_float4(__uint_as_float(r[4 * j]), __uint_as_float(r[4 * j + 1]), __uint_as_float(r[4 * j + 2]),
+                           __uint_as_float(r[4 * j + 3]));
+    } else {
+#pragma unroll
+      for (int j = 0; j < 32; ++j)
+        if (col + j < N) d0[j] = __uint_as_float(r[j]);
+    }
+  }
+};
+
+// The exact FP64 value of an FP32 one, and min(max(z, lo), hi), on the integer pipe: on GB300 the
+// conversion and the FP64 min/max issue on the FP64 pipe (1.7 lanes/clk/SM).  Zeros, subnormals,
+// infinities and NaN take the instructions, in functions of their own: inlined, the compiler runs
+// them for every element and selects (measured: the decoder at 444 us instead of its rate below).
+__device__ __noinline__ double widen_rare(uint32_t b) { return (double)__uint_as_float(b); }
+__device__ __noinline__ double clip_rare(double z, double lo, double hi) { return fmin(fmax(z, lo), hi); }
+__device__ __forceinline__ double widen(uint32_t b) {
+  const uint32_t e = (b >> 23) & 0xffu;
+  if (e - 1u >= 254u) return widen_rare(b);
+  return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20))), (int)(b << 29));
+}
+// monotone map of the non-NaN doubles onto signed integers, and back
+__device__ __forceinline__ long long order(double a) {
+  const long long b = __double_as_longlong(a);
+  return b ^ ((b >> 63) & 0x7fffffffffffffffll);
+}
+// (by halves: masking the sign of the whole word is compiled to an FP64 absolute value)
+__device__ __forceinline__ bool is_nan(double a) {
+  const unsigned h = (unsigned)__double2hiint(a) & 0x7fffffffu;
+  return h + (__double2loint(a) != 0 ? 1u : 0u) > 0x7ff00000u;
+}
+
+// Z[col][row] = clip(mu[row] + alpha acc, lo[row], hi[row]) in FP64: the decoder of the learned start.
+// A warp's 32 lanes hold 32 consecutive rows of one column, so the stores of Z are coalesced without
+// a transpose and the FP32 product never goes to memory.  One FP64 operation per element (19 SM
+// cycles per warp) bounds it at 72 us for 150,000 x 256, beside the 45 us that writing Z's
+// 307 MB takes; three CTAs per SM overlap the FP64 epilogue of one with the short K loops of the
+// others.  150,000 x 256, K = 256: 155 us, against 309 us for a separate decoder kernel behind a
+// 100 us product.
+struct EpiDecode {
+  double alpha;
+  const double *mu, *lo, *hi;
+  double* Z;
+  int64_t ldz;
+  static constexpr int kStages = 2, kBlocks = 3;
+  struct Row {
+    double mu;
+    long long lo, hi;   // order() of the bounds
+    bool rare;          // a bound is NaN
+  };
+  __device__ __forceinline__ Row row(int i) const {
+    return Row{mu[i], order(lo[i]), order(hi[i]), is_nan(lo[i]) || is_nan(hi[i])};
+  }
+  __device__ __forceinline__ void operator()(const Row& q, int, int row, int col, int N,
+                                             const uint32_t (&r)[32]) const {
+    double* d = Z + (int64_t)col * ldz + row;
+#pragma unroll
+    for (int j = 0; j < 32; ++j)
+      if (col + j < N) {
+        const double z = fma(alpha, widen(r[j]), q.mu);
+        if (q.rare || is_nan(z)) {
+          d[j * ldz] = clip_rare(z, lo[row], hi[row]);
+        } else {
+          long long k = order(z);
+          k = k < q.lo ? q.lo : k;
+          k = k > q.hi ? q.hi : k;
+          d[j * ldz] = __longlong_as_double(k ^ ((k >> 63) & 0x7fffffffffffffffll));
+        }
+      }
+  }
+};
+
+template <int BN, class Epi>
+__global__ void __launch_bounds__(128, Epi::kBlocks)
+    k_gemm_bf16(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb, const Epi epi, int M,
+                int N, int kb_total, int kb_per) {
   static_assert(BN == 64 || BN == 128 || BN == 256, "TMEM columns must be a power of two >= 32");
+  static_assert(BN * Epi::kBlocks <= 512, "the resident CTAs share 512 TMEM columns");
+  constexpr int kStages = Epi::kStages;
   constexpr uint32_t kBTile = (uint32_t)BN * kBK * 2;
   __shared__ __align__(8) uint64_t bar_full[kStages];
   __shared__ __align__(8) uint64_t bar_empty[kStages];
@@ -204,25 +293,14 @@ __global__ void __launch_bounds__(128, 1)
   tc_fence_after();
   if (ok) {
     const int row = m0 + warp * 32 + lane;
-    float* crow = C + (int64_t)blockIdx.z * split_stride + (int64_t)row * ldc;
+    typename Epi::Row q = {};
+    if (row < M) q = epi.row(row);
 #pragma unroll 1
     for (int c0 = 0; c0 < BN; c0 += 32) {
       uint32_t r[32];
       tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, r);
       const int col = n0 + c0;
-      if (row < M && col < N) {
-        if (vec && col + 32 <= N) {
-          float4* d = reinterpret_cast<float4*>(crow + col);
-#pragma unroll
-          for (int j = 0; j < 8; ++j)
-            d[j] = make_float4(__uint_as_float(r[4 * j]), __uint_as_float(r[4 * j + 1]),
-                               __uint_as_float(r[4 * j + 2]), __uint_as_float(r[4 * j + 3]));
-        } else {
-#pragma unroll
-          for (int j = 0; j < 32; ++j)
-            if (col + j < N) crow[col + j] = __uint_as_float(r[j]);
-        }
-      }
+      if (row < M && col < N) epi(q, (int)blockIdx.z, row, col, N, r);
     }
   }
   tc_fence_before();
@@ -274,19 +352,28 @@ cudaError_t make_map(CUtensorMap* map, const void* ptr, int64_t rows, int64_t co
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-template <int BN>
-cudaError_t launch(const CUtensorMap& ta, const CUtensorMap& tb, float* C, int64_t ldc, int64_t split_stride,
-                   int64_t M, int64_t N, int kb_total, int kb_per, int splits, int vec, cudaStream_t s) {
-  constexpr uint32_t bytes = smem_bytes<BN>();
+template <int BN, class Epi>
+cudaError_t launch(const CUtensorMap& ta, const CUtensorMap& tb, const Epi& epi, int64_t M, int64_t N, int kb_total,
+                   int kb_per, int splits, cudaStream_t s) {
+  constexpr uint32_t bytes = smem_bytes<BN, Epi::kStages>();
   static std::once_flag once;
   static cudaError_t attr = cudaSuccess;
   std::call_once(once, [] {
-    attr = cudaFuncSetAttribute(k_gemm_bf16<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    attr = cudaFuncSetAttribute(k_gemm_bf16<BN, Epi>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   });
   if (attr != cudaSuccess) return attr;
   dim3 grid((unsigned)((M + kBM - 1) / kBM), (unsigned)((N + BN - 1) / BN), (unsigned)splits);
-  k_gemm_bf16<BN><<<grid, 128, bytes, s>>>(ta, tb, C, ldc, split_stride, (int)M, (int)N, kb_total, kb_per, vec);
+  k_gemm_bf16<BN, Epi><<<grid, 128, bytes, s>>>(ta, tb, epi, (int)M, (int)N, kb_total, kb_per);
   return cudaGetLastError();
+}
+
+// The operand checks that every product shares; what is wrong, or null.
+const char* check_operands(int64_t M, int64_t N, int64_t K, const void* A, int64_t lda, const void* B, int64_t ldb) {
+  if (!A || !B) return "A or B is null";
+  if (lda < K || ldb < K) return "lda and ldb must be >= K";
+  if (lda % 8 || ldb % 8) return "lda and ldb must be multiples of 8 (16-byte rows)";
+  if ((reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(B)) & 15) return "A and B must be 16-byte aligned";
+  return nullptr;
 }
 
 }  // namespace
@@ -308,10 +395,7 @@ cudaError_t gemm_bf16(int64_t M, int64_t N, int64_t K, const void* A, int64_t ld
     }
     return cudaSuccess;
   }
-  if (!A || !B) return bad("A or B is null");
-  if (lda < K || ldb < K) return bad("lda and ldb must be >= K");
-  if (lda % 8 || ldb % 8) return bad("lda and ldb must be multiples of 8 (16-byte rows)");
-  if ((reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(B)) & 15) return bad("A and B must be 16-byte aligned");
+  if (const char* w = check_operands(M, N, K, A, lda, B, ldb)) return bad(w);
   const int kb_total = (int)((K + kBK - 1) / kBK);
   splits = std::max(1, std::min(splits, kb_total));
   const int kb_per = (kb_total + splits - 1) / splits;
@@ -328,14 +412,35 @@ cudaError_t gemm_bf16(int64_t M, int64_t N, int64_t K, const void* A, int64_t ld
   float* out = splits > 1 ? work : C;
   const int64_t ld = splits > 1 ? N : ldc;
   const int vec = ((reinterpret_cast<uintptr_t>(out) & 15) == 0 && ld % 4 == 0) ? 1 : 0;
-  e = BN == 64    ? launch<64>(ta, tb, out, ld, M * N, M, N, kb_total, kb_per, splits, vec, stream)
-      : BN == 128 ? launch<128>(ta, tb, out, ld, M * N, M, N, kb_total, kb_per, splits, vec, stream)
-                  : launch<256>(ta, tb, out, ld, M * N, M, N, kb_total, kb_per, splits, vec, stream);
+  const EpiStore epi{out, ld, M * N, vec};
+  e = BN == 64    ? launch<64>(ta, tb, epi, M, N, kb_total, kb_per, splits, stream)
+      : BN == 128 ? launch<128>(ta, tb, epi, M, N, kb_total, kb_per, splits, stream)
+                  : launch<256>(ta, tb, epi, M, N, kb_total, kb_per, splits, stream);
   if (e != cudaSuccess || splits == 1) return e;
   const int64_t total = M * N;
   const int blocks = (int)std::min<int64_t>((total + 255) / 256, 152 * 16);
   k_splitk_sum<<<blocks, 256, 0, stream>>>(work, splits, M, N, C, ldc);
   return cudaGetLastError();
+}
+
+cudaError_t gemm_decode(int64_t D, int64_t N, int64_t K, const void* A, int64_t lda, const void* B, int64_t ldb,
+                        double alpha, const double* mu, const double* lo, const double* hi, double* Z, int64_t ldz,
+                        cudaStream_t stream, const char** why) {
+  auto bad = [why](const char* w) {
+    if (why) *why = w;
+    return cudaErrorInvalidValue;
+  };
+  if (D < 1 || N < 1 || K < 1 || D >= (1ll << 31) || N > 65535ll * 64 || K >= (1ll << 31)) return bad("size out of range");
+  if (const char* w = check_operands(D, N, K, A, lda, B, ldb)) return bad(w);
+  // the tile width of gemm_bf16 up to 128 columns (256 would leave room for two CTAs per SM only)
+  const int BN = N <= 64 ? 64 : 128;
+  const int kb = (int)((K + kBK - 1) / kBK);
+  CUtensorMap ta, tb;
+  cudaError_t e;
+  if ((e = make_map(&ta, A, D, K, lda, kBM)) != cudaSuccess) return e;
+  if ((e = make_map(&tb, B, N, K, ldb, BN)) != cudaSuccess) return e;
+  const EpiDecode epi{alpha, mu, lo, hi, Z, ldz};
+  return BN == 64 ? launch<64>(ta, tb, epi, D, N, kb, kb, 1, stream) : launch<128>(ta, tb, epi, D, N, kb, kb, 1, stream);
 }
 
 int gemm_error_flag() {

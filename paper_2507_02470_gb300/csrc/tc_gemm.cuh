@@ -20,6 +20,12 @@ namespace tc {
 cudaError_t gemm_bf16(int64_t M, int64_t N, int64_t K, const void* A, int64_t lda, const void* B, int64_t ldb,
                       float* C, int64_t ldc, int splits, float* work, cudaStream_t stream, const char** why);
 
+// Z[n][i] = clip(mu[i] + alpha (A B^T)[i][n], lo[i], hi[i]) in FP64 for A (D x K) and B (N x K) as
+// above, in one launch: the FP32 product stays in tensor memory.  Z is N x D with leading dimension ldz.
+cudaError_t gemm_decode(int64_t D, int64_t N, int64_t K, const void* A, int64_t lda, const void* B, int64_t ldb,
+                        double alpha, const double* mu, const double* lo, const double* hi, double* Z, int64_t ldz,
+                        cudaStream_t stream, const char** why);
+
 // Reads and clears the device flag that a GEMM kernel sets when one of its bounded waits
 // gave up (0: none; 1 producer, 2 MMA issuer, 3 epilogue).  Synchronises the device.
 int gemm_error_flag();
