@@ -173,10 +173,10 @@ typedef struct hprqp_params {
                                 formed directly instead of by the Halpern recurrence of its
                                 image (rounding only).  0: every step runs all five passes */
   int32_t factor_inline;     /* factor terms B_f^T B_f without a tiled copy: 1 (default) a thin
-                                factor (sum over B's rows of their squared lengths <= n / 2)
-                                has the inner step's products t = B x formed inside the Q row
-                                pass from B's rows, with no separate pre-pass launch; 2: every
-                                such factor; 0: never.  Sums in another order (rounding only) */
+                                factor (sum over B's rows of their squared lengths <= n / 2) is
+                                multiplied in the inner step through the explicit entries of its
+                                B^T B, with no separate pre-pass launch; 2: every such factor (up
+                                to 1e9 entries); 0: never.  Sums in another order (rounding only) */
   int32_t wait_polls;        /* launch_mode 3: polls of one grid-barrier wait before the solve
                                 gives up with HPRQP_TIMEOUT; 0 (default): about a second */
   int32_t batch_team;        /* batched solver: 0 (default) threads per instance chosen per bucket

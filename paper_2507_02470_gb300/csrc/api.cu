@@ -19,6 +19,7 @@
 
 #include "../../include/hprqp.h"
 #include "../../include/hprqp_learn.h"
+#include "resident.cuh"
 #include "sell_build.cuh"
 #include "solver.cuh"
 
@@ -57,6 +58,11 @@ struct hprqp_handle {
   Ctrl* hctrl2 = nullptr;     // pinned mirror
   cudaStream_t pstream = nullptr;
   cudaEvent_t pfork = nullptr, pjoin = nullptr;
+  // resident solver (resident.cu): its plan (B = 0: not used), barrier flags, partial sums, results
+  ResPlan res;
+  unsigned* res_flags = nullptr;
+  double *res_part = nullptr, *res_lam = nullptr;
+  double pw_start[2] = {0.0, 0.0};   // 1 / ||start vector|| of the power methods, once computed
   cudaEvent_t ev[2] = {nullptr, nullptr};
   std::string err;
   hprqp_kkt kkt;
@@ -576,6 +582,140 @@ struct PhaseClock {
   }
 };
 
+
+// ------------------------------------------------------------------------------------ resident plan
+// Most entries of rows [b R + at, (b + 1) R + at) of a matrix over the blocks b, by its row pointers
+// (at: where its first row lies in the numbering that is split)
+static int64_t most_entries(const std::vector<int>& rp, int64_t rows, int64_t R, int64_t at = 0) {
+  int64_t most = 0;
+  for (int64_t lo = at / R * R; lo < at + rows; lo += R) {
+    const int64_t q0 = std::max<int64_t>(lo - at, 0), q1 = std::min<int64_t>(lo + R - at, rows);
+    most = std::max<int64_t>(most, rp[q1] - rp[q0]);
+  }
+  return most;
+}
+static std::vector<int> column_pointers(const HostCsr& M) {
+  std::vector<int> cp(M.cols + 1, 0);
+  for (int j : M.ci) cp[j + 1]++;
+  for (int64_t j = 0; j < M.cols; j++) cp[j + 1] += cp[j];
+  return cp;
+}
+
+// Splits the problem over blocks for the resident solver and lays out their shared memory (p.B stays
+// 0 when it does not apply).  It takes what needs no more than the state in shared memory: matrices
+// that do not fit beside it are read through L2.  Options that ask for a schedule of the separate
+// kernels (launch_mode, fixed_schedule, fused_steps, pdl, autotune, factor_inline, tiled_factor other than their
+// defaults) get that schedule.
+static hprqp_status plan_resident(hprqp_handle* h, const HostCsr& A, const HostCsr& qcsr, const HostCsr& thin,
+                                  const std::vector<HostCsr>& facs, int sms) {
+  const hprqp_params& q = h->prm;
+  const QDev& Q = h->args.Q;
+  ResPlan p;
+  if (q.launch_mode != 0 || q.method != 0 || !q.fixed_schedule || !q.fused_steps || !q.pdl || q.autotune != 1 ||
+      q.factor_inline != 1 || q.tiled_factor != 1 || !Q.present() || Q.qap_d)
+    return HPRQP_OK;
+  for (int f = 0; f < Q.nfac; f++)
+    if (Q.tiled[f]) return HPRQP_OK;
+  int coop = 0, optin = 0;
+  CU(h, cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, h->dev));
+  CU(h, cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->dev));
+  if (!coop) return HPRQP_OK;
+  const int64_t n = h->n, m = h->m;
+  int64_t frows = 0, fnnz = 0, drows = 0;
+  for (auto& B : facs) {
+    frows += B.rows;
+    fnnz += B.rp[B.rows];
+  }
+  for (int g = 0; g < Q.ndense; g++) drows += Q.dense_p[g];
+  const int64_t annz = m > 0 ? A.rp[m] : 0, qnnz = qcsr.rows ? qcsr.rp[n] : 0;
+  const int64_t room = (optin - (int64_t)resident_static_smem() - 512) / (int64_t)sizeof(double);
+  // Blocks of about 64 rows of R^n, fewer rows where the products are long.  One cluster (16 blocks at most)
+  // while that asks for no more than 32 blocks and the copies of the gathered vectors leave half of the
+  // shared memory; measured, us per step in a cluster / on a grid: n = 1000 (Q = M^T M) 15.0 / 18.6, 2500
+  // 14.3 / 15.9, 4000 17.6 / 16.2, 10,000 18.7 / 9.8; dense factor n = 700 20.7 / 22.1, 1500 32.6 / 26.7.
+  const int64_t by_rows = (n + 63) / 64, by_work = (2 * annz + 2 * fnnz + qnnz) / 1024 + drows * n / 2048;
+  const int64_t blocks = std::max<int64_t>(1, std::max(by_rows, by_work)), copies = 3 * n + 2 * m + 3 * Q.tlen;
+  int cl = 1;
+  while (cl < 16 && cl < blocks) cl *= 2;
+  p.cluster = by_rows <= 40 && by_work <= 32 && copies + (int64_t)kResStateN * ((n + cl - 1) / cl) <= room / 2;
+  p.B = p.cluster ? cl : (int)std::min<int64_t>(sms, blocks);
+  p.rn = (int)((n + p.B - 1) / p.B);
+  if (!p.cluster) p.B = (int)((n + p.rn - 1) / p.rn);
+  p.rm = (int)((m + p.B - 1) / p.B);
+  p.rp = (int)std::max<int64_t>(1, (frows + p.B - 1) / p.B);
+  p.rd = (int)std::max<int64_t>(1, (drows + p.B - 1) / p.B);
+  // threads: idle warps only lengthen the block's barriers, more than the rows need is no gain
+  p.T = p.rn > 512 ? 1024 : p.rn > 256 || drows * n > 200000 ? 512 : 256;
+  // lanes per row: no more than the row has entries, nor than the block has threads for its rows
+  auto lanes = [&](int64_t rows, int64_t nnz, int64_t own) {
+    if (rows == 0) return 1;
+    const int64_t avg = nnz / rows;
+    if (avg >= 512 && own <= 4) return 0;
+    int g = 1;
+    while (g < 32 && 2 * g <= avg && 2 * g * own <= p.T) g *= 2;
+    return g;
+  };
+  p.gA = lanes(m, annz, p.rm);
+  p.gAT = lanes(n, annz, p.rn);
+  p.gQ = lanes(n, qnnz, p.rn);
+  p.gT = thin.rp.empty() ? 1 : lanes(n, thin.rp[n], p.rn);
+  p.gF = lanes(n, fnnz, p.rn);
+  p.gP = lanes(frows, fnnz, p.rp);
+  p.cw = 32;
+  while (p.cw < p.rn && p.cw < p.T) p.cw *= 2;
+  for (int f = 0; f < Q.nfac; f++) p.pre |= !Q.inl[f];
+  p.pre |= Q.ndense > 0;
+  p.rs_len = std::max(p.rn, p.rm);
+  int64_t at = (int64_t)kResStateN * p.rn + (int64_t)kResStateM * p.rm;
+  p.o_rs = (int)at;
+  at += 2 * p.rs_len;
+  p.o_scratch = (int)at;
+  at += 4 * p.T;
+  p.o_vec = (int)at;
+  if (p.cluster) at += copies + 2 * p.B * 16;
+  if (at > room) return HPRQP_OK;
+  auto take = [&](int64_t len) -> int {   // len doubles, or -1 when they do not fit
+    if (len > room - at) return -1;
+    const int o = (int)at;
+    at += len;
+    return o;
+  };
+  auto place = [&](ResPlan::M& M, int64_t nnz, int64_t rows) {
+    const int64_t li = (nnz + 1) / 2, lr = (rows + 2) / 2;
+    const int o = take(nnz + li + lr);
+    if (o < 0) return;
+    M.o_v = o;
+    M.o_ci = o + (int)nnz;
+    M.o_rp = o + (int)(nnz + li);
+  };
+  if (m > 0) {
+    place(p.A, most_entries(A.rp, m, p.rm), p.rm);
+    place(p.AT, most_entries(column_pointers(A), n, p.rn), p.rn);
+  }
+  if (qcsr.rows) place(p.Qc, most_entries(qcsr.rp, n, p.rn), p.rn);
+  if (!thin.rp.empty()) place(p.thin, most_entries(thin.rp, n, p.rn), p.rn);
+  for (int f = 0; f < Q.nfac; f++) {
+    place(p.fact[f], most_entries(column_pointers(facs[f]), n, p.rn), p.rn);
+    if (!Q.inl[f]) place(p.fac[f], most_entries(facs[f].rp, facs[f].rows, p.rp, Q.toff[f]), p.rp);
+  }
+  if (Q.diag) p.o_diag = take(p.rn);
+  for (int k = 0; k < Q.ndia; k++) p.o_dia[k] = take((int64_t)p.rn + Q.dia_off[k]);
+  for (int g = 0; g < Q.ndense; g++) {
+    p.o_dcol[g] = take(Q.dense_p[g] * p.rn);
+    p.o_drow[g] = take((int64_t)p.rd * n);
+  }
+  p.smem = (size_t)at * sizeof(double);
+  if (!resident_fits(p, sms)) return HPRQP_OK;
+  void* d;
+  hprqp_status st;
+  if ((st = dalloc(h, &d, 2 * sizeof(unsigned)))) return st;
+  h->res_flags = (unsigned*)d;
+  if ((st = zeros(h, &h->res_part, (size_t)2 * p.B * 16))) return st;
+  if ((st = zeros(h, &h->res_lam, 2))) return st;
+  h->res = p;
+  return HPRQP_OK;
+}
+
 static hprqp_status create_impl(hprqp_handle* h, int64_t n, int64_t m, const hprqp_qop* Q, const int32_t* A_rowptr,
                                 const int32_t* A_colidx, const double* A_vals, const double* c, const double* l,
                                 const double* u, const double* L, const double* U, int32_t phi, double lambda) {
@@ -896,19 +1036,48 @@ static hprqp_status create_impl(hprqp_handle* h, int64_t n, int64_t m, const hpr
     }
     if (any) CU(h, tiled_setup());
   }
-  // ---- thin factor terms: the inner step forms (B x)_r inside the Q row pass from row r of B.
-  // The extra gathers per row of Q are sum_r len(r)^2 / n (every entry of B^T's row j re-reads
-  // a whole row of B); at most 1/2 per row the pass saves the pre-pass launch and its latency
-  // (S of the n = 1e6 CQP: 1e4 rows of 3, 0.09 per row)
-  for (int f = 0; f < QD.nfac; f++) {
-    if (QD.tiled[f] || h->prm.factor_inline == 0) continue;
-    const HostCsr& B = facs[f];
-    double sq = 0.0;
-    for (int64_t r = 0; r < B.rows; r++) {
-      const double len = (double)(B.rp[r + 1] - B.rp[r]);
-      sq += len * len;
+  // ---- thin factor terms: the inner step multiplies with the explicit entries of B^T B (sum_r len(r)^2 of
+  // them); at most n / 2 they cost less than the pre-pass launch and its latency (S of the n = 1e6 CQP: 1e4
+  // rows of 3, 9e4 entries)
+  HostCsr thin;
+  {
+    thin.rows = thin.cols = n;
+    double pairs = 0.0;   // entries of all thin terms: 32-bit row pointers
+    for (int f = 0; f < QD.nfac; f++) {
+      if (QD.tiled[f] || h->prm.factor_inline == 0) continue;
+      const HostCsr& B = facs[f];
+      double sq = 0.0;
+      for (int64_t r = 0; r < B.rows; r++) {
+        const double l = (double)(B.rp[r + 1] - B.rp[r]);
+        sq += l * l;
+      }
+      if (sq > 0.5 * (double)n && h->prm.factor_inline != 2) continue;
+      if (pairs + sq > 1e9) continue;
+      pairs += sq;
+      QD.inl[f] = 1;
+      if (thin.rp.empty()) thin.rp.assign(n + 1, 0);
+      for (int64_t r = 0; r < B.rows; r++)
+        for (int k = B.rp[r]; k < B.rp[r + 1]; k++) thin.rp[B.ci[k] + 1] += B.rp[r + 1] - B.rp[r];
     }
-    if (h->prm.factor_inline == 2 || sq <= 0.5 * (double)n) QD.inl[f] = 1;
+    if (!thin.rp.empty()) {
+      for (int64_t j = 0; j < n; j++) thin.rp[j + 1] += thin.rp[j];
+      thin.ci.resize(thin.rp[n]);
+      thin.v.resize(thin.rp[n]);
+      std::vector<int> at(thin.rp.begin(), thin.rp.end() - 1);
+      for (int f = 0; f < QD.nfac; f++) {
+        if (!QD.inl[f]) continue;
+        const HostCsr& B = facs[f];
+        for (int64_t r = 0; r < B.rows; r++)
+          for (int k = B.rp[r]; k < B.rp[r + 1]; k++) {
+            int& q = at[B.ci[k]];
+            for (int i = B.rp[r]; i < B.rp[r + 1]; i++, q++) {
+              thin.ci[q] = B.ci[i];
+              thin.v[q] = B.v[k] * B.v[i];
+            }
+          }
+      }
+      if ((st = upload_csr(h, QD.thin, thin))) return st;
+    }
   }
   QD.tlen = toff;
 
@@ -1019,7 +1188,7 @@ static hprqp_status create_impl(hprqp_handle* h, int64_t n, int64_t m, const hpr
     CU(h, cudaEventCreateWithFlags(&h->pjoin, cudaEventDisableTiming));
     h->pw_pair = true;
   }
-  CU(h, cudaMallocHost(&h->hflags, 8 * sizeof(int)));
+  CU(h, cudaMallocHost(&h->hflags, 16 * sizeof(int)));   // done flags; two doubles from word 8 on
   CU(h, cudaEventCreate(&h->ev[0]));
   CU(h, cudaEventCreate(&h->ev[1]));
   CU(h, cudaStreamSynchronize(h->stream));
@@ -1071,6 +1240,7 @@ static hprqp_status create_impl(hprqp_handle* h, int64_t n, int64_t m, const hpr
     // plain steps of the fixed-schedule graph end with the fused passes (need Q and A)
     P.fuse = (h->prm.fused_steps != 0 && QD.present() && m > 0) ? 1 : 0;
   }
+  if ((st = plan_resident(h, A, qcsr, thin, facs, sms))) return st;
   clk.mark("autotune");
   return HPRQP_OK;
 }
@@ -1319,20 +1489,65 @@ static hprqp_status build_pw_graph(hprqp_handle* h, int which) {
   return HPRQP_OK;
 }
 
+// 1 / ||start vector|| of the power method on R^m (which = 0) or R^n, same start vector and summation
+// order as the CPU reference; it depends on the size alone, so a handle computes it once
+static double power_start_scale(hprqp_handle* h, int which) {
+  double& v = h->pw_start[which];
+  if (v == 0.0) {
+    const int64_t dim = which == 0 ? h->m : h->n;
+    double s2 = 0.0;
+    for (int64_t i = 0; i < dim; i++) {
+      const uint32_t hh = (uint32_t)((uint64_t)(i + 1) * 2654435761u);
+      const double x = 0.5 + (double)hh / 4294967296.0;
+      s2 += x * x;
+    }
+    v = 1.0 / std::sqrt(s2);
+  }
+  return v;
+}
+
+static ResRun resident_run(const hprqp_handle* h, long long steps) {
+  ResRun r;
+  r.steps = steps;
+  r.flags = h->res_flags;
+  r.err = reinterpret_cast<int*>(h->res_flags + 1);
+  r.part = h->res_part;
+  r.lam = h->res_lam;
+  return r;
+}
+
+// The power methods that `which` asks for (bit 0: A A^*, bit 1: Q) in one launch of the resident form.
+static hprqp_status resident_power(hprqp_handle* h, int which, double* lamA, double* lamQ) {
+  Range rg("hprqp_power_resident");
+  ResPower pw;
+  if (which & 1) {
+    pw.va = h->pwA_args.V.pv;
+    pw.wa = h->pwA_args.V.pw;
+    pw.u = h->pwA_args.V.ptmp;
+    pw.scale[0] = power_start_scale(h, 0);
+  }
+  if (which & 2) pw.scale[1] = power_start_scale(h, 1);
+  pw.tol = h->prm.power_tol;
+  pw.max_iter = h->prm.power_max_iter;
+  const ResRun r = resident_run(h, 0);
+  CU(h, launch_resident_power(h->args, h->res, r, which, pw, h->stream));
+  h->launches += 1;
+  double* lam = reinterpret_cast<double*>(h->hflags + 8);
+  CU(h, cudaMemcpyAsync(lam, h->res_lam, 2 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+  CU(h, cudaMemcpyAsync(h->hflags, r.err, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+  CU(h, cudaStreamSynchronize(h->stream));
+  if (h->hflags[0]) return fail(h, HPRQP_TIMEOUT, "resident power method: a grid barrier wait gave up");
+  if (which & 1) *lamA = h->prm.power_safety * lam[0];
+  if (which & 2) *lamQ = h->prm.power_safety * lam[1];
+  return HPRQP_OK;
+}
+
 // Power method of Sec. 4.1 on A A^* (which = 0, R^m) or Q (which = 1, R^n); returns the
 // Rayleigh quotient at convergence times the safety factor.
 static hprqp_status power_method(hprqp_handle* h, int which, double* lam) {
   Range rg(which == 0 ? "hprqp_power_A" : "hprqp_power_Q");
-  const int64_t dim = which == 0 ? h->m : h->n;
   hprqp_status st;
   if ((st = build_pw_graph(h, which))) return st;
-  // host value of 1/||start||, same start vector and summation order as the CPU reference
-  double s2 = 0.0;
-  for (int64_t i = 0; i < dim; i++) {
-    uint32_t hh = (uint32_t)((uint64_t)(i + 1) * 2654435761u);
-    double v = 0.5 + (double)hh / 4294967296.0;
-    s2 += v * v;
-  }
   // with the paired state (m > 0 and Q present), the method on A A^* keeps to its own
   // controller copy and vectors, as its graph does, also when it runs alone
   const bool pair = which == 0 && h->pw_pair;
@@ -1343,7 +1558,7 @@ static hprqp_status power_method(hprqp_handle* h, int which, double* lam) {
   C.pw_it = 0;
   C.pw_lam = 0.0;
   C.pw_done = 0;
-  C.pw_scale = 1.0 / std::sqrt(s2);
+  C.pw_scale = power_start_scale(h, which);
   C.pw_max = h->prm.power_max_iter;
   C.pw_tol = h->prm.power_tol;
   C.done = 1;  // keep the iteration kernels idle
@@ -1376,16 +1591,6 @@ static hprqp_status power_both(hprqp_handle* h, double* lamA, double* lamQ) {
   if ((st = build_pw_graph(h, 0))) return st;
   if ((st = build_pw_graph(h, 1))) return st;
   const Args pa = pw_pair_args(h);
-  auto start_scale = [](int64_t dim) {
-    // host value of 1/||start||, same start vector and summation order as the CPU reference
-    double s2 = 0.0;
-    for (int64_t i = 0; i < dim; i++) {
-      uint32_t hh = (uint32_t)((uint64_t)(i + 1) * 2654435761u);
-      double v = 0.5 + (double)hh / 4294967296.0;
-      s2 += v * v;
-    }
-    return 1.0 / std::sqrt(s2);
-  };
   Ctrl* hc[2] = {h->hctrl2, h->hctrl};
   Ctrl* dc[2] = {h->dctrl2, h->dctrl};
   cudaStream_t ss[2] = {h->pstream, h->stream};
@@ -1397,7 +1602,7 @@ static hprqp_status power_both(hprqp_handle* h, double* lamA, double* lamQ) {
     C.pw_it = 0;
     C.pw_lam = 0.0;
     C.pw_done = 0;
-    C.pw_scale = start_scale(w == 0 ? h->m : h->n);
+    C.pw_scale = power_start_scale(h, w);
     C.pw_max = h->prm.power_max_iter;
     C.pw_tol = h->prm.power_tol;
     C.done = 1;  // keep the iteration kernels idle
@@ -1768,6 +1973,29 @@ static hprqp_status solve_persist(hprqp_handle* h, std::chrono::steady_clock::ti
   return finish_solve(h, t0, t1, lamA, lamQ, sigma, time_up);
 }
 
+// Algorithm 4 in launches of the resident solver: one launch runs to the end of the solve (at most
+// 2^15 steps), or one check period at a time where a time limit is to be kept.
+static hprqp_status solve_resident(hprqp_handle* h, std::chrono::steady_clock::time_point t0,
+                                   std::chrono::steady_clock::time_point t1, double lamA, double lamQ, double sigma) {
+  const bool limited = h->prm.time_limit > 0;
+  const ResRun r = resident_run(h, limited ? std::min<int64_t>(h->prm.check_every, 1024) : 1 << 15);
+  bool time_up = false;
+  for (;;) {
+    CU(h, launch_resident(h->args, h->res, r, h->stream));
+    h->launches += 1;
+    CU(h, cudaMemcpyAsync(&h->hflags[0], &h->dctrl->done, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+    CU(h, cudaMemcpyAsync(&h->hflags[1], r.err, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+    CU(h, cudaStreamSynchronize(h->stream));
+    if (h->hflags[1]) return fail(h, HPRQP_TIMEOUT, "resident solver: a grid barrier wait gave up");
+    if (h->hflags[0]) break;
+    if (limited && std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count() > h->prm.time_limit) {
+      time_up = true;
+      break;
+    }
+  }
+  return finish_solve(h, t0, t1, lamA, lamQ, sigma, time_up);
+}
+
 extern "C" hprqp_status hprqp_solve(hprqp_handle* h, double tol, int64_t max_iter) {
   if (!h) return HPRQP_INVALID_ARG;
   h->err.clear();
@@ -1781,7 +2009,13 @@ extern "C" hprqp_status hprqp_solve(hprqp_handle* h, double tol, int64_t max_ite
   h->fixed_steps = 0;
   // ---- lambda_A >= lambda_1(AA^*), lambda_Q >= lambda_1(Q) (Sec. 4.1)
   double lamA = 0.0, lamQ = 0.0;
-  if (HA && HQ && h->pw_pair && !(h->prm.lambda_A > 0) && !(h->prm.lambda_Q > 0)) {
+  if (h->res.B) {
+    const int need = (HA && !(h->prm.lambda_A > 0) ? 1 : 0) | (HQ && !(h->prm.lambda_Q > 0) ? 2 : 0);
+    if (need && (st = resident_power(h, need, &lamA, &lamQ))) return st;
+    if (HA && !(need & 1)) lamA = h->prm.lambda_A;
+    if (HQ && !(need & 2)) lamQ = h->prm.lambda_Q;
+    if (HA && !(lamA > 0.0)) lamA = 1.0;
+  } else if (HA && HQ && h->pw_pair && !(h->prm.lambda_A > 0) && !(h->prm.lambda_Q > 0)) {
     if ((st = power_both(h, &lamA, &lamQ))) return st;
     if (!(lamA > 0.0)) lamA = 1.0;
   } else {
@@ -1807,6 +2041,7 @@ extern "C" hprqp_status hprqp_solve(hprqp_handle* h, double tol, int64_t max_ite
   Range rg("hprqp_iterate");
   if (h->prm.launch_mode == 2) return solve_stream(h, t0, t1, lamA, lamQ, sigma);
   if (h->prm.launch_mode == 3) return solve_persist(h, t0, t1, lamA, lamQ, sigma);
+  if (h->res.B) return solve_resident(h, t0, t1, lamA, lamQ, sigma);
   bool time_up = false;
   // ---- Algorithm 4 in launches of the fixed-schedule graph while fixed_L steps remain
   build_fixed(h);

@@ -401,6 +401,7 @@ __device__ void solve_one(const Pools& P, int idx, Shared<PC>& S) {
     C.ttest = (1 % C.check_every == 0) || (1 >= C.max_iter);
     C.status = 1;
     set_sigma(C, sigma);
+    halpern_weights(C, C.fha, C.fhb);
   }
   __syncthreads();
 

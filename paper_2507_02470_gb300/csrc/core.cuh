@@ -90,10 +90,11 @@ struct QDev {
   // stopping test keep the CSR pre-pass and row pass
   int tiled[kMaxFac] = {0};
   // thin factor terms (few rows of B meet any row of B^T: sum over B's rows of their squared
-  // lengths is small against n): the inner step's products form (B x)_r from row r of B inside
-  // the row pass that needs it, with no pre-pass; other products (apply, power method, restart
-  // difference) still use the pre-pass
+  // lengths is small against n): the inner step and the power method multiply with the explicit
+  // entries of their B^T B, kept as one CSR matrix `thin`, with no pre-pass; other products (apply,
+  // restart difference) still use the pre-pass
   int inl[kMaxFac] = {0};
+  Csr thin;                              // rows == 0: absent
   TiledFac tf[kMaxFac];
   int64_t uoff[kMaxFac] = {0};
   int64_t tfd = 0;              // intermediate rows of the factor and dense terms

@@ -71,30 +71,11 @@ __device__ __forceinline__ int stream_i32(const int* p, const L2Pol& q) {
 }
 #endif
 
-// The value a CSR pass multiplies entry (i, c) with: the c-th element of a vector in memory, or,
-// for a thin factor term B (see QDev::inl), (B x)_c formed from row c of B on demand (entries
-// in stored order), so that the pass needs no pre-pass writing t = B x first.
+// The value a CSR pass multiplies entry (i, c) with: the c-th element of a vector in memory.
 struct GatherX {
   const double* p;
   __device__ __forceinline__ double operator()(int c, const L2Pol& pol) const { return gather_f64(p + c, pol); }
 };
-struct FacRowX {
-  const int* rp;
-  const int* ci;
-  const double* v;
-  const double* x;
-  __device__ __forceinline__ double operator()(int c, const L2Pol& pol) const {
-    const int b = rp[c], e = rp[c + 1];
-    double s = 0.0;
-    for (int k = b; k < e; k++) s = fma(v[k], gather_f64(x + ci[k], pol), s);
-    return s;
-  }
-};
-
-template <class X>
-constexpr bool kOnDemand = false;
-template <>
-constexpr bool kOnDemand<FacRowX> = true;
 
 // Conditional-node handles set by the controller (graph mode); zero flags when unused.
 struct Handles {
@@ -188,17 +169,7 @@ __device__ __forceinline__ void csr_chunk_lanes(const Csr& M, int64_t row0, cons
   for (int rr = grp; rr < kChunk; rr += NG) {
     const int64_t row = row0 + rr;
     double s0 = 0.0, s1 = 0.0;
-    if (row < M.rows && kOnDemand<X0>) {
-      // values formed on demand (thin factor): rows of B^T hold a few entries at most, so one
-      // entry at a time, with no unrolled loads to keep in registers
-      const int b = stream_i32(M.rp + row, pol), e = stream_i32(M.rp + row + 1, pol);
-      for (int k = b + lane; k < e; k += G) {
-        const int c = stream_i32(M.ci + k, pol);
-        const double v = stream_f64(M.v + k, pol);
-        s0 = fma(v, x0(c, pol), s0);
-        if (NR == 2) s1 = fma(v, x1(c, pol), s1);
-      }
-    } else if (row < M.rows) {
+    if (row < M.rows) {
       const int b = stream_i32(M.rp + row, pol), e = stream_i32(M.rp + row + 1, pol);
       int k = b + lane;
       for (; k + 3 * G < e; k += 4 * G) {
@@ -388,8 +359,9 @@ __device__ __forceinline__ void csr_chunk(const Csr& M, int64_t row0, const doub
 }
 
 // All CSR-like parts of Q (explicit CSR and every B_f^T with its intermediate t_f) for a chunk.
-// inl: the pass belongs to an inner step, where a thin factor term (Q.inl) forms t_f = B_f x on
-// demand from B_f's rows (x = x0, and x1 for the second vector) instead of reading t.
+// inl: the pass belongs to an inner step, where the thin factor terms (Q.inl) are multiplied by the
+// explicit entries of their B^T B instead of reading t (rp -> entry -> x where B^T, t formed from B's
+// rows, took rp -> row of B -> entry -> x, and a quarter fewer FP64 instructions).
 template <int G, int NR>
 __device__ __forceinline__ void q_csr_chunk(const QDev& Q, int64_t row0, const double* x0, const double* x1,
                                             const double* t0, const double* t1, double* rs0, double* rs1,
@@ -399,14 +371,14 @@ __device__ __forceinline__ void q_csr_chunk(const QDev& Q, int64_t row0, const d
     csr_chunk<G, NR>(Q.csr, row0, x0, x1, rs0, rs1, false);
     add = true;
   }
+  if (inl && Q.thin.rows) {
+    csr_chunk<G, NR>(Q.thin, row0, x0, x1, rs0, rs1, add);
+    add = true;
+  }
   for (int f = 0; f < Q.nfac; f++) {
     if (NR == 1 && Q.tiled[f]) continue;   // B_f^T t_f formed by the tiled kernels (q_local)
-    if (inl && Q.inl[f]) {
-      const Csr& B = Q.fac[f];
-      csr_chunk_x<G, NR>(Q.fact[f], row0, FacRowX{B.rp, B.ci, B.v, x0}, FacRowX{B.rp, B.ci, B.v, x1}, rs0, rs1, add);
-    } else {
-      csr_chunk<G, NR>(Q.fact[f], row0, t0 + Q.toff[f], NR == 2 ? t1 + Q.toff[f] : nullptr, rs0, rs1, add);
-    }
+    if (inl && Q.inl[f]) continue;
+    csr_chunk<G, NR>(Q.fact[f], row0, t0 + Q.toff[f], NR == 2 ? t1 + Q.toff[f] : nullptr, rs0, rs1, add);
     add = true;
   }
   if (!add) {
@@ -571,8 +543,8 @@ __device__ __forceinline__ void pre_body(const Args& a, int which) {
       if (r < ffac)
         while (term + 1 < Q.nfac && r >= Q.toff[term + 1]) term++;
       // one-vector products of a tiled factor are formed by the tiled kernels; the products of
-      // a thin factor for an inner step or the power method are formed inside the row pass
-      // (q_csr_chunk)
+      // a thin factor for an inner step or the power method come from its explicit B^T B in the
+      // row pass (q_csr_chunk)
       const bool step_src = which == PRE_WH || which == PRE_WB || which == PRE_W || which == PRE_PV;
       const bool mine = r < ffac && !(Q.tiled[term] && !two) && !(Q.inl[term] && step_src);
       if (mine) {
@@ -765,7 +737,8 @@ __device__ __forceinline__ void controller(Ctrl& C, const double* Ls, const doub
     C.t = 0;
     C.r++;
   } else {
-    halpern_weights(C, C.ha, C.hb);
+    C.ha = C.fha;   // set with t and k of this step
+    C.hb = C.fhb;
     C.mode = 1;
     C.t++;
   }
@@ -1118,6 +1091,67 @@ __device__ __forceinline__ void sigma_argmin_dev(double t1, double t2, double t3
   *out = exp(0.5 * (A + B));
 }
 
+// The exact minimiser of eq. (3.12) by one warp (valid in every lane): the bracket of
+// sigma_argmin_dev, cut into 33 parts per round.  The sign of f' is taken from f' sigma^2
+// (1 + lQ sigma)^2, which needs no division: a dozen rounds of about ten FP64 operations, where the
+// bisection by one thread took 70 us (50 rounds of three dependent divisions).
+__device__ __forceinline__ double sigma_argmin_warp(double t1, double t2, double t3, double lq) {
+  const int lane = threadIdx.x & 31;
+  double hi = sqrt(t2 / t1);
+  if (t3 <= 0.0 || lq <= 0.0) return hi;
+  double lo = sqrt(t2 / (t1 + t3 / lq));
+  const double f = (double)(lane + 1) * (1.0 / 33.0);
+  for (int it = 0; it < 64 && (hi - lo) > 4.0e-16 * hi; it++) {
+    const double mid = fma(hi - lo, f, lo);
+    const double d = fma(lq, mid, 1.0), m2 = mid * mid;
+    const double g = fma(fma(t1, m2, -t2) * d, d, t3 * m2 * mid * (1.0 + d));
+    const unsigned up = __ballot_sync(0xffffffffu, g > 0.0);
+    const int first = up ? __ffs(up) - 1 : 32;   // the root lies below this lane's point
+    const double nhi = first < 32 ? __shfl_sync(0xffffffffu, mid, first & 31) : hi;
+    const double nlo = first > 0 ? __shfl_sync(0xffffffffu, mid, (first + 31) & 31) : lo;
+    if (nhi == hi && nlo == lo) break;
+    hi = nhi;
+    lo = nlo;
+  }
+  return 0.5 * (lo + hi);
+}
+
+// Algorithm 5 by one warp: theta~ of eq. (3.11) from the sums |dy|^2, <dw, Q dw>, <Q dw, d>, |dx|^2,
+// <d, Q d> (d = A^* dy; the same in every lane), floors, argmin of eq. (3.12), smoothing.
+__device__ __forceinline__ void algorithm5(Ctrl& C, double dy2, double wqw, double qwd, double dx2, double th3) {
+  const double th1 = fmax(C.lamA * dy2 + C.lamQ * wqw - 2.0 * qwd, 1e-12);
+  const double th2 = fmax(dx2, 1e-12);
+  double snew;
+  if (C.sigma_golden) sigma_argmin_dev(th1, th2, th3, C.lamQ, 1, &snew);
+  else snew = sigma_argmin_warp(th1, th2, th3, C.lamQ);
+  const int lane = threadIdx.x & 31;
+  const double beta = exp(-C.ratio);
+  const double lg = log(lane == 0 ? snew : C.sigma);   // both logarithms at once
+  const double sig = exp(beta * __shfl_sync(0xffffffffu, lg, 0) + (1.0 - beta) * __shfl_sync(0xffffffffu, lg, 1));
+  // set_sigma's quotients, one per lane: 1/sigma, c1, c2, s, 1/(sigma lambda_A)
+  const double d = 1.0 + sig * C.lamQ, slA = sig * C.lamA;
+  const double q = (lane == 1 ? sig * C.lamQ : lane == 3 ? sig : 1.0) / (lane == 0 ? sig : lane == 4 ? (slA > 0.0 ? slA : 1.0) : d);
+  const double c1 = __shfl_sync(0xffffffffu, q, 1), c2 = __shfl_sync(0xffffffffu, q, 2), s = __shfl_sync(0xffffffffu, q, 3),
+               islA = __shfl_sync(0xffffffffu, q, 4);
+  __syncwarp();
+  if (lane == 0) {
+    if (!isfinite(sig) || !(sig > 0.0)) {
+      C.status = 3;
+      C.done = 1;
+    } else {
+      C.sigma = sig;
+      C.inv_sigma = q;
+      C.c1 = c1;
+      C.c2 = c2;
+      C.s = s;
+      C.slA = slA;
+      C.inv_slA = slA > 0.0 ? islA : 0.0;
+      C.tau = sig * C.lambda;
+    }
+    C.restart_pending = 0;
+  }
+}
+
 template <int G>
 __device__ __forceinline__ void restart_body(const Args& a) {
   Ctrl* HPRQP_RESTRICT C = a.C;
@@ -1199,24 +1233,10 @@ __device__ __forceinline__ void restart_body(const Args& a) {
   if (!last_block(&a.counters[1])) return;
   double tot[kWR];
   reduce_partials<kWR>(a.partR, gridDim.x, kWR, 0u, tot, red);
-  if (threadIdx.x == 0) {
-    // Algorithm 5: theta~ of eq. (3.11), floors, argmin of eq. (3.12), smoothing
-    double th1 = C->lamA * tot[0] + C->lamQ * tot[1] - 2.0 * tot[2];
-    double th2 = tot[3];
-    const double th3 = tot[4];
-    th1 = fmax(th1, 1e-12);
-    th2 = fmax(th2, 1e-12);
-    double snew;
-    sigma_argmin_dev(th1, th2, th3, C->lamQ, C->sigma_golden, &snew);
-    const double beta = exp(-C->ratio);
-    const double sig = exp(beta * log(snew) + (1.0 - beta) * log(C->sigma));
-    if (!isfinite(sig) || !(sig > 0.0)) {
-      C->status = 3;
-      C->done = 1;
-    } else {
-      set_sigma(*C, sig);
-    }
-    C->restart_pending = 0;
+  if (threadIdx.x < 32) {   // thread 0 holds the sums
+#pragma unroll
+    for (int i = 0; i < kWR; i++) tot[i] = __shfl_sync(0xffffffffu, tot[i], 0);
+    algorithm5(*C, tot[0], tot[1], tot[2], tot[3], tot[4]);
   }
 }
 

@@ -81,12 +81,13 @@ struct Plan {
 };
 
 // Halpern weights 1/(i+2), (i+1)/(i+2) of the step after the current one (Algorithm 4; i the
-// inner counter t, or k with halpern_total), evaluated before the controller advances t and k.
-// The controller and the fused passes use this one expression, so their weights agree bit for bit.
+// inner counter t, or k with halpern_total), evaluated when t and k are set; the controller takes
+// them over as ha, hb when the step ends, so its weights and the fused passes' agree bit for bit.  One
+// division: on GB300 a dependent FP64 division takes 640 cycles, on the critical path of every step.
 __host__ __device__ inline void halpern_weights(const Ctrl& C, double& ha, double& hb) {
   const double i = C.halpern_total ? (double)C.k : (double)C.t;
   ha = 1.0 / (i + 2.0);
-  hb = (i + 1.0) / (i + 2.0);
+  hb = 1.0 - ha;
 }
 
 // sigma and the scalars derived from it (host and device use the same arithmetic)
