@@ -19,6 +19,7 @@
 
 #include "../../include/hprqp.h"
 #include "../../include/hprqp_learn.h"
+#include "qap_tc.cuh"
 #include "resident.cuh"
 #include "sell_build.cuh"
 #include "solver.cuh"
@@ -59,6 +60,7 @@ struct hprqp_handle {
   cudaStream_t pstream = nullptr;
   cudaEvent_t pfork = nullptr, pjoin = nullptr;
   // resident solver (resident.cu): its plan (B = 0: not used), barrier flags, partial sums, results
+  QapTc* qap_tc = nullptr;   // tensor-core form of the QAP term
   ResPlan res;
   unsigned* res_flags = nullptr;
   double *res_part = nullptr, *res_lam = nullptr;
@@ -406,6 +408,7 @@ static void release(hprqp_handle* h) {
   if (h->hctrl) cudaFreeHost(h->hctrl);
   if (h->hctrl2) cudaFreeHost(h->hctrl2);
   if (h->hflags) cudaFreeHost(h->hflags);
+  if (h->qap_tc) qap_tc_free(h->qap_tc);
   if (h->side) cudaStreamDestroy(h->side);
   if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
   cudaGetLastError();
@@ -424,10 +427,10 @@ extern "C" hprqp_status hprqp_memory_stats(const hprqp_handle* h, int64_t* out) 
 }
 
 // ------------------------------------------------------------------------------------ autotune
-static int tune_G(hprqp_handle* h, const Csr& M, int grid, double* x, double* y, int fallback) {
+static int tune_G(hprqp_handle* h, const Csr& M, int R, int grid, double* x, double* y, int fallback) {
   if (M.rows == 0 || M.nnz == 0) return fallback;
   if (h->prm.autotune == 2) return 0;
-  if (h->prm.autotune == 3) return M.soff ? -1 : 1;
+  if (h->prm.autotune == 3) return M.soff && R == kChunk ? -1 : 1;
   if (!h->prm.autotune) {
     double avg = (double)M.nnz / (double)M.rows;
     return avg < 6 ? 1 : avg < 12 ? 2 : avg < 24 ? 4 : avg < 64 ? 8 : 32;
@@ -438,12 +441,13 @@ static int tune_G(hprqp_handle* h, const Csr& M, int grid, double* x, double* y,
   float best = 1e30f;
   int bestG = fallback;
   for (int G : cand) {
-    if (G == -1 && !M.soff) continue;
-    launch_spmv_probe(M, G, grid, x, y, h->stream);
+    if (G == -1 && (!M.soff || R != kChunk)) continue;
+    if (G == 2 && R != kChunk) continue;   // eight rows at two lanes are half a warp: its shuffles take all lanes
+    launch_spmv_probe(M, G, R, grid, x, y, h->stream);
     float tot = 0;
     for (int r = 0; r < 3; r++) {
       cudaEventRecord(h->ev[0], h->stream);
-      launch_spmv_probe(M, G, grid, x, y, h->stream);
+      launch_spmv_probe(M, G, R, grid, x, y, h->stream);
       cudaEventRecord(h->ev[1], h->stream);
       cudaEventSynchronize(h->ev[1]);
       float ms = 0;
@@ -492,6 +496,10 @@ static hprqp_status data_norms(hprqp_handle* h, const std::vector<double>& hc, c
   h->c_inf = ci;
   return HPRQP_OK;
 }
+
+// Size from which the QAP product runs on the tensor cores (autotune = 1): its five launches take 43 us where
+// the two FP64 contractions take 49 at d = 9 and 85 at d = 32
+constexpr int64_t kQapTcMinD = 8;
 
 // Scratch of the QAP term's split contractions (qap.cu): partial tiles and per-tile counters
 static hprqp_status qap_scratch(hprqp_handle* h, QDev& QD) {
@@ -1008,7 +1016,15 @@ static hprqp_status create_impl(hprqp_handle* h, int64_t n, int64_t m, const hpr
     QD.qap_in = qin;
     QD.qap_off = toff;
     toff += n;
-    if ((st = qap_scratch(h, QD))) return st;
+    if (qap_d >= kQapTcMinD && h->prm.autotune == 1) {
+      size_t parts[5];
+      void* mem;
+      if ((st = dalloc(h, &mem, qap_tc_bytes(qap_d, parts)))) return st;
+      CU(h, qap_tc_create(&h->qap_tc, qap_d, QD.qap, mem, h->stream));
+      QD.qap_tc = h->qap_tc;
+    } else if ((st = qap_scratch(h, QD))) {
+      return st;
+    }
   }
   clk.mark("device problem");
   // ---- tiled copies of large factor terms: their one-vector products gather through shared
@@ -1113,7 +1129,10 @@ static hprqp_status create_impl(hprqp_handle* h, int64_t n, int64_t m, const hpr
   auto chunks = [](int64_t rows) { return (int)std::max<int64_t>(1, (rows + kChunk - 1) / kChunk); };
   const int per_sm = 4;
   P.gridN = std::min(chunks(n), sms * per_sm);
-  P.gridM = std::min(chunks(m), sms * per_sm);
+  // few long rows of A (QAP d = 256: 512 rows of 256 entries): eight rows a block, so that they spread over
+  // the SMs (two blocks of 256 rows took 67 us, as long as both Q products of a step now do)
+  a.rowsA = h->prm.launch_mode != 3 && m > 0 && chunks(m) < sms && a.A.nnz / m >= 32 ? 8 : kChunk;
+  P.gridM = (int)std::min<int64_t>(std::max<int64_t>(1, (m + a.rowsA - 1) / a.rowsA), sms * per_sm);
   P.gridE = std::min(chunks(n), sms * 8);
   P.gridT = tiled_tbt_grid(n, sms);
   P.gridPre = (int)std::min<int64_t>(std::max<int64_t>(1, (toff + 7) / 8), sms * 8);
@@ -1197,13 +1216,13 @@ static hprqp_status create_impl(hprqp_handle* h, int64_t n, int64_t m, const hpr
   // ---- schedule autotune (lanes per row for each CSR pass)
   {
     CU(h, cudaMemsetAsync(ain, 0, nm * sizeof(double), h->stream));
-    P.gA = m > 0 ? tune_G(h, a.A, P.gridM, ain, aout, 1) : 1;
-    P.gAT = m > 0 ? tune_G(h, a.AT, P.gridN, ain, aout, 1) : 1;
+    P.gA = m > 0 ? tune_G(h, a.A, a.rowsA, P.gridM, ain, aout, 1) : 1;
+    P.gAT = m > 0 ? tune_G(h, a.AT, kChunk, P.gridN, ain, aout, 1) : 1;
     const Csr* big = nullptr;
     if (QD.csr.rows) big = &QD.csr;
     for (int f = 0; f < QD.nfac; f++)
       if (!big || QD.fact[f].nnz > big->nnz) big = &QD.fact[f];
-    P.gQ = big ? tune_G(h, *big, P.gridN, ain, aout, 1) : 1;
+    P.gQ = big ? tune_G(h, *big, kChunk, P.gridN, ain, aout, 1) : 1;
     // Q's CSR-like parts are only thin factors formed on demand: one lane per row (their few
     // entries gain nothing from more lanes, and the bare-SpMV probe cannot see the on-demand
     // products).  A SELL copy of B^T, which packs a chunk's entries into one warp, measured
@@ -1634,6 +1653,15 @@ static hprqp_status power_both(hprqp_handle* h, double* lamA, double* lamQ) {
   *lamA = h->prm.power_safety * h->hctrl2->pw_lam;
   *lamQ = h->prm.power_safety * h->hctrl->pw_lam;
   return HPRQP_OK;
+}
+
+// A bounded wait of the tensor-core QAP kernels that gave up since the handle was created (the caller has
+// nothing in flight on the stream, or waits for it here)
+static hprqp_status qap_check(hprqp_handle* h) {
+  if (!h->qap_tc) return HPRQP_OK;
+  CU(h, cudaMemcpyAsync(&h->hflags[4], qap_tc_error(h->qap_tc), sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+  CU(h, cudaStreamSynchronize(h->stream));
+  return h->hflags[4] ? fail(h, HPRQP_TIMEOUT, "QAP product: a tensor-core kernel gave up a bounded wait") : HPRQP_OK;
 }
 
 // ------------------------------------------------------------------------------------ solve
@@ -2095,6 +2123,7 @@ static hprqp_status finish_solve(hprqp_handle* h, std::chrono::steady_clock::tim
   Ctrl& C = *h->hctrl;
   CU(h, cudaMemcpyAsync(h->hctrl, h->dctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, h->stream));
   CU(h, cudaStreamSynchronize(h->stream));
+  if (const hprqp_status qs = qap_check(h)) return qs;
   auto t2 = std::chrono::steady_clock::now();
   int status = C.status;
   if (!C.done) status = time_up ? HPRQP_TIME_LIMIT : HPRQP_MAX_ITER;
@@ -2288,5 +2317,5 @@ extern "C" hprqp_status hprqp_apply(hprqp_handle* h, int32_t op, const double* i
   if (h->scaled) CU(h, launch_vmul(V.aout, op == 0 ? V.ise : V.isd, nout, h->stream));
   CU(h, cudaMemcpyAsync(out, V.aout, nout * sizeof(double), cudaMemcpyDefault, h->stream));
   CU(h, cudaStreamSynchronize(h->stream));
-  return HPRQP_OK;
+  return qap_check(h);
 }

@@ -58,6 +58,8 @@ struct TiledFac {
   double* part = nullptr;         // b.ntile x p partial sums of B x, one row per column tile
 };
 
+struct QapTc;
+
 // Q = diag(d) + sym band + CSR + sum_f B_f^T B_f + sum_g F_g^T F_g   (Sec. 1: Q may be
 // matrix-free).  The factor intermediates t = B v, F v live in one buffer at toff[].
 struct QDev {
@@ -84,6 +86,7 @@ struct QDev {
   double* qap_part = nullptr;   // qap_splits x d x d partial tiles of a split contraction
   unsigned* qap_count = nullptr;   // one counter per 32 x 32 tile of the result
   int qap_splits = 1;           // blocks sharing the K range of one tile
+  const QapTc* qap_tc = nullptr;   // host object of the tensor-core form (qap_tc.cu), or null
   int64_t qap_off = 0;
   // factor terms with a tiled copy: their one-vector products (t = B x, then u = B^T t into
   // the intermediate buffer at uoff) run in the tiled kernels; the two-vector products of a
@@ -177,13 +180,16 @@ __device__ __forceinline__ bool iisinf(double a) {
 }
 
 // ---------------------------------------------------------------------------- block reductions
-// Deterministic: fixed lane/warp order.  op 0 = sum, 1 = max of non-negative values.
+// Deterministic: fixed lane/warp order.  op 0 = sum, 1 = max of non-negative values; terms outside `want`
+// are left alone (a term costs five FP64 instructions per warp).
 template <int NT>
-__device__ __forceinline__ void block_reduce(double (&v)[NT], const unsigned maxmask, double* smem) {
+__device__ __forceinline__ void block_reduce(double (&v)[NT], const unsigned maxmask, double* smem,
+                                             const unsigned want = 0xffffffffu) {
   // smem: at least NT * 32 doubles
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
 #pragma unroll
   for (int i = 0; i < NT; i++) {
+    if (!((want >> i) & 1u)) continue;
     double a = v[i];
     bool mx = (maxmask >> i) & 1u;
 #pragma unroll
@@ -197,6 +203,7 @@ __device__ __forceinline__ void block_reduce(double (&v)[NT], const unsigned max
   if (warp == 0) {
 #pragma unroll
     for (int i = 0; i < NT; i++) {
+      if (!((want >> i) & 1u)) continue;
       bool mx = (maxmask >> i) & 1u;
       double a = lane < nw ? smem[i * 32 + lane] : 0.0;
 #pragma unroll
@@ -230,17 +237,19 @@ __device__ __forceinline__ bool last_block(unsigned* counter) {
 // the block takes part; the result is valid in out[] of thread 0.  Fixed order.
 template <int NT>
 __device__ __forceinline__ void reduce_partials(const double* part, int nblocks, int W, unsigned maxmask,
-                                                double (&out)[NT], double* smem) {
+                                                double (&out)[NT], double* smem,
+                                                const unsigned want = 0xffffffffu) {
 #pragma unroll
   for (int i = 0; i < NT; i++) out[i] = 0.0;
   for (int b = threadIdx.x; b < nblocks; b += blockDim.x) {
 #pragma unroll
     for (int i = 0; i < NT; i++) {
+      if (!((want >> i) & 1u)) continue;
       double p = __ldcg(part + (size_t)b * W + i);
       out[i] = ((maxmask >> i) & 1u) ? imax(out[i], p) : out[i] + p;
     }
   }
-  block_reduce<NT>(out, maxmask, smem);
+  block_reduce<NT>(out, maxmask, smem, want);
 }
 
 }  // namespace hprqp

@@ -157,16 +157,16 @@ __device__ __forceinline__ double conj_phi_term(int phi, double z, double L, dou
 }
 
 // ------------------------------------------------------------------------------------ CSR pass
-// Row sums of a chunk of kChunk rows, G lanes per row, into shared rs0/rs1 (add: accumulate).
+// Row sums of a chunk of R rows, G lanes per row, into shared rs0/rs1 (add: accumulate).
 template <int G, int NR, class X0, class X1>
 __device__ __forceinline__ void csr_chunk_lanes(const Csr& M, int64_t row0, const X0& x0, const X1& x1, double* rs0,
-                                                double* rs1, bool add) {
+                                                double* rs1, bool add, int R) {
   const int lane = threadIdx.x % G;
   const int grp = threadIdx.x / G;
   constexpr int NG = kThreads / G;
   const L2Pol pol;
 #pragma unroll 1
-  for (int rr = grp; rr < kChunk; rr += NG) {
+  for (int rr = grp; rr < R; rr += NG) {   // (R a multiple of the rows of a warp)
     const int64_t row = row0 + rr;
     double s0 = 0.0, s1 = 0.0;
     if (row < M.rows) {
@@ -239,14 +239,14 @@ __device__ __forceinline__ void csr_chunk_lanes(const Csr& M, int64_t row0, cons
 constexpr int kWin = 1024;
 template <int NR, class X0, class X1>
 __device__ __forceinline__ void csr_chunk_staged(const Csr& M, int64_t row0, const X0& x0, const X1& x1, double* rs0,
-                                                 double* rs1, bool add) {
+                                                 double* rs1, bool add, int R) {
   __shared__ int srp[kChunk + 1];
   __shared__ double sv[kWin];
   __shared__ double sx[NR][kWin];
   constexpr int kPer = kWin / kThreads;
   const int t = threadIdx.x;
   const L2Pol pol;
-  const int nr = (int)(M.rows - row0 < (int64_t)kChunk ? M.rows - row0 : (int64_t)kChunk);
+  const int nr = (int)(M.rows - row0 < (int64_t)R ? M.rows - row0 : (int64_t)R);
   if (nr <= 0) return;   // block-uniform: no row of this matrix in the chunk
   __syncthreads();   // an earlier pass over this chunk may still read srp, sv, sx
   for (int i = t; i <= nr; i += kThreads) srp[i] = stream_i32(M.rp + row0 + i, pol);
@@ -342,20 +342,21 @@ __device__ __forceinline__ void csr_chunk_sell(const Csr& M, int64_t row0, const
 // where G asks for the SELL form.
 template <int G, int NR, class X0, class X1>
 __device__ __forceinline__ void csr_chunk_x(const Csr& M, int64_t row0, const X0& x0, const X1& x1, double* rs0,
-                                            double* rs1, bool add) {
+                                            double* rs1, bool add, int R) {
   if constexpr (G == 0) {
-    csr_chunk_staged<NR>(M, row0, x0, x1, rs0, rs1, add);
+    csr_chunk_staged<NR>(M, row0, x0, x1, rs0, rs1, add, R);
   } else if constexpr (G == -1) {
     if (M.soff) csr_chunk_sell<NR>(M, row0, x0, x1, rs0, rs1, add);
-    else csr_chunk_lanes<1, NR>(M, row0, x0, x1, rs0, rs1, add);
+    else csr_chunk_lanes<1, NR>(M, row0, x0, x1, rs0, rs1, add, R);
   } else {
-    csr_chunk_lanes<G, NR>(M, row0, x0, x1, rs0, rs1, add);
+    csr_chunk_lanes<G, NR>(M, row0, x0, x1, rs0, rs1, add, R);
   }
 }
 template <int G, int NR>
 __device__ __forceinline__ void csr_chunk(const Csr& M, int64_t row0, const double* HPRQP_RESTRICT x0,
-                                          const double* HPRQP_RESTRICT x1, double* rs0, double* rs1, bool add) {
-  csr_chunk_x<G, NR>(M, row0, GatherX{x0}, GatherX{x1}, rs0, rs1, add);
+                                          const double* HPRQP_RESTRICT x1, double* rs0, double* rs1, bool add,
+                                          int R = kChunk) {
+  csr_chunk_x<G, NR>(M, row0, GatherX{x0}, GatherX{x1}, rs0, rs1, add, R);
 }
 
 // All CSR-like parts of Q (explicit CSR and every B_f^T with its intermediate t_f) for a chunk.
@@ -804,10 +805,11 @@ __device__ __forceinline__ void end_row(EndTerms& T, const Args& a, int64_t j, b
 
 // Reduce the end terms of this block, elect the last block, run the controller.
 template <bool ACTIVE>
-__device__ __forceinline__ void end_iteration(EndTerms& T, const Args& a, const Handles& hd, bool active) {
+__device__ __forceinline__ void end_iteration(EndTerms& T, const Args& a, const Handles& hd, bool active,
+                                              unsigned want) {
   __shared__ double red[kWL * 32];
   if (ACTIVE && active) {
-    block_reduce<kWL>(T.s, kEndMax, red);
+    block_reduce<kWL>(T.s, kEndMax, red, want);
     if (threadIdx.x == 0) {
 #pragma unroll
       for (int i = 0; i < kWL; i++) a.partL[(size_t)blockIdx.x * kWL + i] = T.s[i];
@@ -820,7 +822,7 @@ __device__ __forceinline__ void end_iteration(EndTerms& T, const Args& a, const 
 #pragma unroll
   for (int i = 0; i < kW3; i++) P3[i] = 0.0;
   if (ACTIVE && active) {
-    reduce_partials<kWL>(a.partL, gridDim.x, kWL, kEndMax, Ls, red);
+    reduce_partials<kWL>(a.partL, gridDim.x, kWL, kEndMax, Ls, red, want);
     __syncthreads();
     if (a.m > 0) reduce_partials<kW3>(a.part3, a.nbM, kW3, 0x6u, P3, red);
   }
@@ -847,7 +849,9 @@ __device__ __forceinline__ void rows_body(const Args& a, const Handles& hd) {
   const bool rtest = (KIND <= K_Q2) ? var_rtest<VAR>(C) : false;
   constexpr bool RED = (VAR != VAR_PLAIN) && !FUSED;   // the variant carries reduction code
   const int64_t rows = (KIND == K_A1 || KIND == K_APPLY_A || KIND == K_POWER_A) ? a.m : a.n;
-  const int64_t nchunks = (rows + kChunk - 1) / kChunk;
+  constexpr bool OVER_M = KIND == K_A1 || KIND == K_APPLY_A || KIND == K_POWER_A;
+  const int R = OVER_M ? a.rowsA : kChunk;
+  const int64_t nchunks = (rows + R - 1) / R;
   const double sigma = C->sigma, s = C->s, slA = C->slA, inv_slA = C->inv_slA;
   const int mode = C->mode;
   // the fused passes apply the Halpern step that follows this one (the weights the controller
@@ -860,7 +864,7 @@ __device__ __forceinline__ void rows_body(const Args& a, const Handles& hd) {
   double pw[kWP] = {0.0, 0.0};
 
   for (int64_t ch = blockIdx.x; ch < nchunks; ch += gridDim.x) {
-    const int64_t row0 = ch * kChunk;
+    const int64_t row0 = ch * R;
     // ---- phase 1: CSR row sums into shared memory
     if (KIND == K_Q1) {
       const double* src = HA ? V.wh : V.wb;
@@ -875,12 +879,12 @@ __device__ __forceinline__ void rows_body(const Args& a, const Handles& hd) {
     } else if (KIND == K_POWER_Q) {
       q_csr_chunk<G, 1>(Q, row0, V.pv, nullptr, V.t1, nullptr, rs0, rs1, true);
     } else if (KIND == K_A1) {
-      if (RED && ttest) csr_chunk<G, 2>(a.A, row0, V.v, V.xb, rs0, rs1, false);
-      else csr_chunk<G, 1>(a.A, row0, V.v, nullptr, rs0, rs1, false);
+      if (RED && ttest) csr_chunk<G, 2>(a.A, row0, V.v, V.xb, rs0, rs1, false, R);
+      else csr_chunk<G, 1>(a.A, row0, V.v, nullptr, rs0, rs1, false, R);
     } else if (KIND == K_APPLY_A) {
-      csr_chunk<G, 1>(a.A, row0, V.ain, nullptr, rs0, rs1, false);
+      csr_chunk<G, 1>(a.A, row0, V.ain, nullptr, rs0, rs1, false, R);
     } else if (KIND == K_POWER_A) {
-      csr_chunk<G, 1>(a.A, row0, V.ptmp, nullptr, rs0, rs1, false);
+      csr_chunk<G, 1>(a.A, row0, V.ptmp, nullptr, rs0, rs1, false, R);
     } else if (KIND == K_AT || KIND == K_ATH) {
       csr_chunk<G, 1>(a.AT, row0, V.yb, nullptr, rs0, rs1, false);
     } else if (KIND == K_APPLY_AT) {
@@ -895,7 +899,7 @@ __device__ __forceinline__ void rows_body(const Args& a, const Handles& hd) {
     if constexpr (G != 1) __syncthreads();
     // ---- phase 2: thread per row, full warps
     const int64_t j = row0 + threadIdx.x;
-    if (j < rows) {
+    if (j < rows && (!OVER_M || (int)threadIdx.x < R)) {
       const double r0 = rs0[threadIdx.x];
       if (KIND == K_Q1) {
         const double* src = HA ? V.wh : V.wb;
@@ -1008,7 +1012,8 @@ __device__ __forceinline__ void rows_body(const Args& a, const Handles& hd) {
       }
     }
   }
-  if (last_of_iter) end_iteration<RED>(T, a, hd, rtest || ttest);
+  // an R~ test needs the first five sums, a stopping test the others
+  if (last_of_iter) end_iteration<RED>(T, a, hd, rtest || ttest, (rtest ? 0x1fu : 0u) | (ttest ? 0xfe0u : 0u));
   if (KIND == K_POWER_Q || KIND == K_POWER_A) {
     __shared__ double redp[kWP * 32];
     block_reduce<kWP>(pw, 0u, redp);

@@ -19,6 +19,7 @@
 #include <vector>
 
 #include "kernels.cuh"
+#include "qap_tc.cuh"
 
 namespace hprqp {
 
@@ -70,6 +71,9 @@ __global__ void k_qap_diff(const double* __restrict__ a, const double* __restric
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += stride) out[i] = a[i] - b[i];
 }
 
+// kernels of one QAP product
+static int qap_kernels(const Args& a) { return !a.Q.qap_d ? 0 : a.Q.qap_tc ? kQapTcKernels : 2; }
+
 cudaError_t launch_qap(const Args& a, const Plan& p, int which, int tt, cudaStream_t s) {
   const QDev& Q = a.Q;
   if (!Q.qap_d) return cudaSuccess;
@@ -83,8 +87,11 @@ cudaError_t launch_qap(const Args& a, const Plan& p, int which, int tt, cudaStre
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
-  cudaError_t e = qap_apply(Q, x, t + Q.qap_off, Q.qap_splits, s);
-  if (e == cudaSuccess && which == 0 && tt != 0) e = qap_apply(Q, V.xb, t + Q.tlen + Q.qap_off, Q.qap_splits, s);
+  auto apply = [&](const double* v, double* out) {
+    return Q.qap_tc ? qap_tc_apply(Q.qap_tc, v, out, s) : qap_apply(Q, v, out, Q.qap_splits, s);
+  };
+  cudaError_t e = apply(x, t + Q.qap_off);
+  if (e == cudaSuccess && which == 0 && tt != 0) e = apply(V.xb, t + Q.tlen + Q.qap_off);
   return e;
 }
 
@@ -178,7 +185,7 @@ cudaError_t launch_step(const Args& a, const Plan& p, cudaStream_t s, int var, c
       L.other();
       const cudaError_t qe = launch_qap(a, p, which, ptt, s);
       if (qe != cudaSuccess) return qe;
-      L.count += 2 + (which == PRE_WH && ptt != 0 ? 2 : 0);
+      L.count += qap_kernels(a) * (which == PRE_WH && ptt != 0 ? 2 : 1);
     }
     return cudaSuccess;
   };
@@ -262,7 +269,7 @@ cudaError_t plan_plain_grids(const Args& a, Plan& p, int sms) {
     const int64_t need = std::max<int64_t>(1, units);
     return (int)std::min<int64_t>(need, (int64_t)sms * occ);
   };
-  const int64_t chN = (a.n + kChunk - 1) / kChunk, chM = (a.m + kChunk - 1) / kChunk;
+  const int64_t chN = (a.n + kChunk - 1) / kChunk, chM = (a.m + a.rowsA - 1) / a.rowsA;
   p.wZX = wave((const void*)zxk(VAR_PLAIN), (a.n + kThreads - 1) / kThreads);
   p.wQ1 = wave((const void*)rowk(K_Q1, VAR_PLAIN, p.gQ), chN);
   p.wQ2 = wave((const void*)rowk(K_Q2, VAR_PLAIN, p.gQ), chN);
@@ -318,7 +325,7 @@ cudaError_t launch_step_fused(const Args& a, const Plan& p, cudaStream_t s, int 
 // kernels before a Q pass of a plain step: the factor pre-pass, the tiled factor kernels and
 // the two contractions of a QAP product
 static int pre_kernels(const Args& a) {
-  return (pre_has_work(a, 1, 0) ? 1 : 0) + 3 * tiled_terms(a) + (a.Q.qap_d ? 2 : 0);
+  return (pre_has_work(a, 1, 0) ? 1 : 0) + 3 * tiled_terms(a) + qap_kernels(a);
 }
 
 int kernels_per_step(const Args& a) {
@@ -331,7 +338,7 @@ int kernels_per_step(const Args& a) {
 }
 int kernels_per_restart(const Args& a) {
   return 1 + ((a.Q.present() && a.m > 0 && a.Q.has_pre())
-                  ? (pre_has_work(a, 2, 0) ? 1 : 0) + 2 * tiled_terms(a) + (a.Q.qap_d ? 3 : 0)
+                  ? (pre_has_work(a, 2, 0) ? 1 : 0) + 2 * tiled_terms(a) + (a.Q.qap_d ? 1 + qap_kernels(a) : 0)
                   : 0);
 }
 int kernels_per_iteration(const Args& a) { return kernels_per_step(a) + kernels_per_restart(a); }
@@ -550,7 +557,7 @@ cudaError_t launch_power_init(const Args& a, const Plan& p, int which, cudaStrea
 
 int kernels_per_power_iter(const Args& a, int which) {
   if (which == 0) return 2;
-  return 1 + (pre_has_work(a, 4, 0) ? 1 : 0) + 3 * tiled_terms(a) + (a.Q.qap_d ? 2 : 0);
+  return 1 + (pre_has_work(a, 4, 0) ? 1 : 0) + 3 * tiled_terms(a) + qap_kernels(a);
 }
 
 // One power iteration, Sec. 4.1: w_{i+1} = M v_i with v_i = w_i / ||w_i||, M = Q or A A^*.  The
@@ -598,15 +605,15 @@ cudaError_t launch_zbar(const Args& a, const Plan& p, cudaStream_t s) {
 
 // plain CSR SpMV used by the schedule autotuner
 template <int G>
-__global__ void __launch_bounds__(kThreads) k_spmv_probe(Csr M, const double* x, double* y) {
+__global__ void __launch_bounds__(kThreads) k_spmv_probe(Csr M, int R, const double* x, double* y) {
   __shared__ double rs0[kChunk];
-  const int64_t nchunks = (M.rows + kChunk - 1) / kChunk;
+  const int64_t nchunks = (M.rows + R - 1) / R;
   for (int64_t ch = blockIdx.x; ch < nchunks; ch += gridDim.x) {
-    const int64_t row0 = ch * kChunk;
-    csr_chunk<G, 1>(M, row0, x, nullptr, rs0, nullptr, false);
+    const int64_t row0 = ch * R;
+    csr_chunk<G, 1>(M, row0, x, nullptr, rs0, nullptr, false, R);
     __syncthreads();
     const int64_t j = row0 + threadIdx.x;
-    if (j < M.rows) y[j] = rs0[threadIdx.x];
+    if ((int)threadIdx.x < R && j < M.rows) y[j] = rs0[threadIdx.x];
     __syncthreads();
   }
 }
@@ -617,16 +624,16 @@ cudaError_t launch_pre_probe(const Args& a, int G, int grid, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_spmv_probe(const Csr& M, int G, int grid, const double* x, double* y, cudaStream_t s) {
+cudaError_t launch_spmv_probe(const Csr& M, int G, int R, int grid, const double* x, double* y, cudaStream_t s) {
   switch (G) {
-    case -1: k_spmv_probe<-1><<<grid, kThreads, 0, s>>>(M, x, y); break;
-    case 0: k_spmv_probe<0><<<grid, kThreads, 0, s>>>(M, x, y); break;
-    case 1: k_spmv_probe<1><<<grid, kThreads, 0, s>>>(M, x, y); break;
-    case 2: k_spmv_probe<2><<<grid, kThreads, 0, s>>>(M, x, y); break;
-    case 4: k_spmv_probe<4><<<grid, kThreads, 0, s>>>(M, x, y); break;
-    case 8: k_spmv_probe<8><<<grid, kThreads, 0, s>>>(M, x, y); break;
-    case 16: k_spmv_probe<16><<<grid, kThreads, 0, s>>>(M, x, y); break;
-    default: k_spmv_probe<32><<<grid, kThreads, 0, s>>>(M, x, y); break;
+    case -1: k_spmv_probe<-1><<<grid, kThreads, 0, s>>>(M, R, x, y); break;
+    case 0: k_spmv_probe<0><<<grid, kThreads, 0, s>>>(M, R, x, y); break;
+    case 1: k_spmv_probe<1><<<grid, kThreads, 0, s>>>(M, R, x, y); break;
+    case 2: k_spmv_probe<2><<<grid, kThreads, 0, s>>>(M, R, x, y); break;
+    case 4: k_spmv_probe<4><<<grid, kThreads, 0, s>>>(M, R, x, y); break;
+    case 8: k_spmv_probe<8><<<grid, kThreads, 0, s>>>(M, R, x, y); break;
+    case 16: k_spmv_probe<16><<<grid, kThreads, 0, s>>>(M, R, x, y); break;
+    default: k_spmv_probe<32><<<grid, kThreads, 0, s>>>(M, R, x, y); break;
   }
   return cudaGetLastError();
 }

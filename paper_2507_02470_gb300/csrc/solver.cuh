@@ -40,6 +40,7 @@ struct Args {
   double* partP;
   unsigned* counters;       // [0] end-of-iteration, [1] restart, [2] power
   int nbM;                  // blocks of the m-row kernel (rows of part3)
+  int rowsA;                // rows of A per block pass of the m-row kernels: kChunk, or fewer (few long rows)
   CheckRec* hist;           // stopping-test records (kHistCap), or null
 };
 
@@ -129,7 +130,7 @@ cudaError_t launch_power_iter(const Args& a, const Plan& p, int which, int i, cu
 int kernels_per_power_iter(const Args& a, int which);
 cudaError_t launch_power_init(const Args& a, const Plan& p, int which, cudaStream_t s);
 cudaError_t launch_zbar(const Args& a, const Plan& p, cudaStream_t s);
-cudaError_t launch_spmv_probe(const Csr& M, int G, int grid, const double* x, double* y, cudaStream_t s);
+cudaError_t launch_spmv_probe(const Csr& M, int G, int R, int grid, const double* x, double* y, cudaStream_t s);
 cudaError_t launch_pre_probe(const Args& a, int G, int grid, cudaStream_t s);
 // shared-memory-tiled factor products (tiled.cu): t = B_f x, then (which != 2) u = B_f^T t,
 // for every tiled factor term; *launched receives the number of kernels
