@@ -8,8 +8,14 @@
 // autotuner picks the block size (64 to 512 threads per instance) and whether a block keeps its
 // instance's dense factor F in shared memory for the whole solve.
 //
-// Per inner step the only work of order k*n is Q xbar-type products through the dense factor
-// (t = F v, then F^T t); everything else is elementwise or of order m*n with m <= 32:
+// Per inner step the only work of order k*n is one product with the transposed dense factor, F^T t, and
+// F xbar; everything else is elementwise or of order m*n with m <= 32:
+//   * t = F wbar_{1/2} is a combination of F xbar, F x and F w (eq. (3.3) is linear in them); the images F x
+//     and F w of the Halpern iterate follow its recurrence, as Q w and A^* y do, with F wbar = F wbar_{1/2} +
+//     s (F A^T)(ybar - y) and F A^T (k x m) formed once per solve;
+//   * F xbar needs only the columns where xbar is not 0.  Under bounds [0, U] most coordinates sit at 0
+//     (portfolio family: 10 to 60 of 5000 do not), so the block lists the others, in order, and gathers
+//     their columns; above n / 8 of them it takes the whole product;
 //   * the second Q product of a step, Q wbar = Q wbar_{1/2} + s (Q A^T)(ybar - y), uses Q A^T
 //     (n x m), formed once per solve (linearity of Q);
 //   * theta_3 of R~ (eq. (2.12)) and theta~_3 of eq. (3.11) are quadratic forms with A Q A^T
@@ -34,6 +40,7 @@ namespace batch {
 
 constexpr int kMaxM = HPRQP_BATCH_MAX_M;
 constexpr int kMaxP = HPRQP_BATCH_MAX_P;
+constexpr int kMaxWarps = 16;   // 512 threads
 
 struct Inst {
   int64_t n, m, p;            // p: rows of the dense factor (0: none)
@@ -44,6 +51,7 @@ struct Inst {
   int64_t oF;                 // offset into the F pool
   int64_t oqat;               // offset into the (n*m) pool
   int64_t oaqa;               // offset into the (m*m) pool
+  int64_t ofat;               // offset into the (p*m) pool
   int64_t oarp, oann;         // A: row pointers (m+1), entries
   int64_t otrp, otnn;         // A^T: row pointers (n+1), entries
   int64_t oqrp, oqnn;         // Q CSR: row pointers (n+1), entries; oqrp < 0: none
@@ -74,7 +82,7 @@ struct Pools {
   const double *l, *u, *y0in;
   double *y, *y0, *yb;
   const double* F;
-  double *qat, *aqa;
+  double *qat, *aqa, *fat;
   const int *arp, *aci, *trp, *tci, *qrp, *qci;
   const double *av, *tv, *qv;
   // algorithm parameters
@@ -98,30 +106,47 @@ __device__ __forceinline__ void bsum(double (&v)[NT], unsigned maxmask, double* 
   __syncthreads();
 }
 
-// t[r] = sum_j F[r][j] x[j] (and F x1 when x1), one warp per row; result in shared t0/t1.  A
-// warp streams one row at a time (consecutive addresses); wider forms that interleave several
-// rows or unroll across rows measured slower on the large instances, whose F comes from HBM.
+// t[r] = sum_j F[r][j] x[j], one warp per row; result in shared t.  A warp streams one row at a time
+// (consecutive addresses), eight loads in flight per lane: one at a time, the rows of a large instance
+// come at the latency of HBM (n = 5000, 16 warps: a millisecond for a product).
 __device__ __forceinline__ void dense_fx(const double* __restrict__ F, int64_t p, int64_t n,
-                                        const double* __restrict__ x0, const double* __restrict__ x1, double* t0,
-                                        double* t1) {
+                                        const double* __restrict__ x, double* t) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   for (int64_t r = warp; r < p; r += nw) {
     const double* Fr = F + r * n;
-    double s0 = 0.0, s1 = 0.0;
-    for (int64_t j = lane; j < n; j += 32) {
-      const double f = Fr[j];
-      s0 = fma(f, x0[j], s0);
-      if (x1) s1 = fma(f, x1[j], s1);
+    double s = 0.0;
+    int64_t j = lane;
+    for (; j + 7 * 32 < n; j += 8 * 32) {
+      double f[8];
+#pragma unroll
+      for (int q = 0; q < 8; q++) f[q] = Fr[j + 32 * q];
+#pragma unroll
+      for (int q = 0; q < 8; q++) s = fma(f[q], x[j + 32 * q], s);
+    }
+    for (; j < n; j += 32) s = fma(Fr[j], x[j], s);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if (lane == 0) t[r] = s;
+  }
+}
+
+// The same from a list of the nz entries of x that are not 0 (their indices and values, in shared memory):
+// eight lanes per row.
+__device__ __forceinline__ void sparse_fx(const double* __restrict__ F, int64_t p, int64_t n,
+                                         const unsigned short* idx, const double* val, int nz, double* t) {
+  const int l = threadIdx.x & 7, grp = threadIdx.x >> 3, ng = blockDim.x >> 3;
+  for (int64_t r0 = 0; r0 < p; r0 += ng) {
+    const int64_t r = r0 + grp;
+    if (r0 + (grp & ~3) >= p) break;   // the whole warp
+    double s = 0.0;
+    if (r < p) {
+      const double* Fr = F + r * n;
+#pragma unroll 4
+      for (int k = l; k < nz; k += 8) s = fma(Fr[idx[k]], val[k], s);
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      s0 += __shfl_down_sync(0xffffffffu, s0, o);
-      if (x1) s1 += __shfl_down_sync(0xffffffffu, s1, o);
-    }
-    if (lane == 0) {
-      t0[r] = s0;
-      if (x1) t1[r] = s1;
-    }
+    for (int o = 4; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o, 8);
+    if (l == 0 && r < p) t[r] = s;
   }
 }
 
@@ -144,7 +169,15 @@ __device__ __forceinline__ double q_row(const Pools& P, const Inst& I, int64_t j
   double acc = 0.0;
   if (I.p) {
     const double* F = fac<FS, PC>(P, I);
-    for (int64_t r = 0; r < I.p; r++) acc = fma(F[r * I.n + j], t[r], acc);
+    int64_t r = 0;
+    for (; r + 7 < I.p; r += 8) {   // eight loads in flight
+      double f[8];
+#pragma unroll
+      for (int q = 0; q < 8; q++) f[q] = F[(r + q) * I.n + j];
+#pragma unroll
+      for (int q = 0; q < 8; q++) acc = fma(f[q], t[r + q], acc);
+    }
+    for (; r < I.p; r++) acc = fma(F[r * I.n + j], t[r], acc);
   }
   if (I.has_diag) acc = fma(P.d[I.on + j], x[j], acc);
   if (I.oqrp >= 0) {
@@ -159,43 +192,59 @@ __device__ __forceinline__ double q_row(const Pools& P, const Inst& I, int64_t j
 // out = Q x for the whole instance (x, out in global memory, x != out); t: shared scratch (p)
 template <bool FS, int PC>
 __device__ void block_qmul(const Pools& P, const Inst& I, const double* x, double* out, double* t) {
-  if (I.p) dense_fx(fac<FS, PC>(P, I), I.p, I.n, x, nullptr, t, nullptr);
+  if (I.p) dense_fx(fac<FS, PC>(P, I), I.p, I.n, x, t);
   __syncthreads();
   for (int64_t j = threadIdx.x; j < I.n; j += blockDim.x) out[j] = q_row<FS, PC>(P, I, j, x, t);
   __syncthreads();
 }
 
-// (A v)_i for all rows i into shared av[m] (and A x1 into ax[m] when x1); block pass over the
-// rows of A: per row, lanes stride its entries, warps combine in shared memory (fixed order)
+// (A v)_i for all rows i into shared av[m] (and A x1 into ax[m] when x1).  The rows are cut into pieces of
+// equal length, about two per warp in all, and a warp sums one piece at a time (fixed order): one
+// reduction over the lanes per piece, where every warp reducing its share of every row issued as many FP64
+// instructions as the rest of a small instance's step.  wred: 2 x kPieces partial sums.
+constexpr int kPieces = kMaxM + 2 * kMaxWarps;   // sum over rows of ceil(len / seg) with seg >= entries / (2 warps)
 __device__ void block_amul(const Pools& P, const Inst& I, const double* __restrict__ v, const double* __restrict__ x1,
                            double* av, double* ax, double* wred) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int* rp = P.arp + I.oarp;
   const int* ci = P.aci + I.oann;
   const double* a = P.av + I.oann;
-  for (int64_t i = 0; i < I.m; i++) {
-    double s0 = 0.0, s1 = 0.0;
-    for (int k = rp[i] + threadIdx.x; k < rp[i + 1]; k += blockDim.x) {
-      const double aik = a[k];
-      s0 = fma(aik, v[ci[k]], s0);
-      if (x1) s1 = fma(aik, x1[ci[k]], s1);
-    }
+  const int m = (int)I.m;
+  const int seg = max(32, (rp[m] + 2 * nw - 1) / (2 * nw));
+  int piece = 0, next = warp;   // pieces before row i; the next one of this warp
+  for (int i = 0; i < m; i++) {
+    const int b = rp[i], e = rp[i + 1], cnt = (e - b + seg - 1) / seg;
+    for (; next < piece + cnt; next += nw) {
+      const int k0 = b + (next - piece) * seg, k1 = min(e, k0 + seg);
+      double s0 = 0.0, s1 = 0.0;
+#pragma unroll 4
+      for (int k = k0 + lane; k < k1; k += 32) {
+        const double aik = a[k];
+        const int j = ci[k];
+        s0 = fma(aik, v[j], s0);
+        if (x1) s1 = fma(aik, x1[j], s1);
+      }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      s0 += __shfl_down_sync(0xffffffffu, s0, o);
-      if (x1) s1 += __shfl_down_sync(0xffffffffu, s1, o);
+      for (int o = 16; o > 0; o >>= 1) {
+        s0 += __shfl_down_sync(0xffffffffu, s0, o);
+        if (x1) s1 += __shfl_down_sync(0xffffffffu, s1, o);
+      }
+      if (lane == 0) {
+        wred[next] = s0;
+        if (x1) wred[kPieces + next] = s1;
+      }
     }
-    if (lane == 0) {
-      wred[i * 32 + warp] = s0;
-      if (x1) wred[(kMaxM + i) * 32 + warp] = s1;
-    }
+    piece += cnt;
   }
   __syncthreads();
-  if (threadIdx.x < I.m) {
+  if ((int)threadIdx.x < m) {
+    int q0 = 0;
+    for (int i = 0; i < (int)threadIdx.x; i++) q0 += (rp[i + 1] - rp[i] + seg - 1) / seg;
+    const int cnt = (rp[threadIdx.x + 1] - rp[threadIdx.x] + seg - 1) / seg;
     double s0 = 0.0, s1 = 0.0;
-    for (int q = 0; q < nw; q++) {
-      s0 += wred[threadIdx.x * 32 + q];
-      if (x1) s1 += wred[(kMaxM + threadIdx.x) * 32 + q];
+    for (int q = q0; q < q0 + cnt; q++) {
+      s0 += wred[q];
+      if (x1) s1 += wred[kPieces + q];
     }
     av[threadIdx.x] = s0;
     if (x1) ax[threadIdx.x] = s1;
@@ -273,12 +322,20 @@ constexpr unsigned kMaxMask = (1u << 5) | (1u << 6) | (1u << 7);
 // t = F v for up to PC factor rows (PC = 256 or HPRQP_BATCH_MAX_P), the m-vectors, the warp
 // partials of a block of at most 16 warps, the controller.  With FS the block's copy of F
 // follows it (dynamic shared memory).
+constexpr int kMaxWords = 512;   // n <= 16,384 for the list of nonzero coordinates
+constexpr int kMaxList = 640;    // n / 8 at n = 5000
 template <int PC>
 struct __align__(16) Shared {
-  double t0[PC], t1[PC];
+  double t0[PC];                                       // F wbar_{1/2} (and scratch)
+  double tx[PC], tx0[PC], txb[PC], tw[PC], tw0[PC], twb[PC];   // F x, F x^{r,0}, F xbar; the same of w
+  unsigned bits[kMaxWords];                            // xbar != 0, by 32 coordinates
+  unsigned short first[kMaxWords];                     // entries of the list before each word
+  unsigned short idx[kMaxList];                        // the coordinates of xbar that are not 0, in order
+  double val[kMaxList];
+  int nz;
   double av[kMaxM], ax[kMaxM];
   double y[kMaxM], yb[kMaxM], y0[kMaxM], lo[kMaxM], hi[kMaxM];
-  double wred[2 * kMaxM * 32];
+  double wred[2 * kPieces];
   double red[kTerms * 32];
   double pm[2][kMaxM];   // power-method vectors on R^m
   Ctrl C;
@@ -300,6 +357,7 @@ __device__ void solve_one(const Pools& P, int idx, Shared<PC>& S) {
   double* ybg = P.yb + I.om;
   double* qat = P.qat + I.oqat;   // [j*m + i] = (Q A^T)_{j i}
   double* aqa = P.aqa + I.oaqa;   // [i*m + l]
+  double* fat = P.fat + I.ofat;   // [r*m + i] = (F A^T)_{r i}
   Ctrl& C = S.C;
   if constexpr (FS) {
     // the block's copy of F, read by every product of the solve
@@ -323,6 +381,7 @@ __device__ void solve_one(const Pools& P, int idx, Shared<PC>& S) {
     __syncthreads();
     block_qmul<FS, PC>(P, I, s1, s2, S.t0);
     for (int64_t j = tid; j < n; j += nt) qat[j * m + i] = s2[j];
+    for (int64_t r = tid; r < I.p; r += nt) fat[r * m + i] = S.t0[r];
     __syncthreads();
   }
   for (int64_t i = 0; i < m; i++) {
@@ -366,6 +425,10 @@ __device__ void solve_one(const Pools& P, int idx, Shared<PC>& S) {
     block_qmul<FS, PC>(P, I, x, Qw, S.t0);
   } else {
     for (int64_t j = tid; j < n; j += nt) Qw[j] = 0.0;
+  }
+  for (int64_t r = tid; r < I.p; r += nt) {
+    const double t = I.has_ws ? S.t0[r] : 0.0;   // F x^0, formed for Q x^0
+    S.tx[r] = S.tx0[r] = S.tw[r] = S.tw0[r] = t;
   }
   for (int64_t j = tid; j < n; j += nt) {
     Qw0[j] = Qw[j];
@@ -412,7 +475,11 @@ __device__ void solve_one(const Pools& P, int idx, Shared<PC>& S) {
     const double sq = C.s, slA = C.slA, islA = C.inv_slA;
     const bool rtest = C.rtest, ttest = C.ttest;
     // P1: Halpern/restart update, eqs. (3.1)-(3.3)
-    for (int64_t j = tid; j < n; j += nt) {
+    const bool listed = I.p > 0 && n <= 32 * kMaxWords;
+    for (int64_t jb = tid & ~31; jb < n; jb += nt) {   // a warp's 32 coordinates at once
+      const int64_t j = jb + (tid & 31);
+      double xbar = 0.0;
+      if (j < n) {
       double xv, wv = 0.0, qw = 0.0, aty = 0.0;
       if (mode == 1) {
         xv = fma(hb, fma(2.0, xb[j], -x[j]), ha * x0[j]);
@@ -454,12 +521,27 @@ __device__ void solve_one(const Pools& P, int idx, Shared<PC>& S) {
       if (HQ) g -= qw;
       if (m > 0) g += aty;
       const double rz = fma(sg, g, xv);
-      const double xbar = prox_phi(I.phi, rz, L[j], U[j], tau);
+      xbar = prox_phi(I.phi, rz, L[j], U[j], tau);
       xb[j] = xbar;
       if (ttest) zb[j] = (xbar - rz) * isg;
       const double xh = fma(2.0, xbar, -xv);
       wh[j] = HQ ? fma(c2, xh, c1 * wv) : 0.0;
       v[j] = xh;   // Q = 0: v = what
+      }
+      if (listed) {
+        const unsigned b = __ballot_sync(0xffffffffu, (__double2hiint(xbar) << 1) != 0 || __double2loint(xbar) != 0);
+        if ((tid & 31) == 0) S.bits[jb >> 5] = b;
+      }
+    }
+    // the images F x, F w of the iterate
+    for (int64_t r = tid; r < I.p; r += nt) {
+      if (mode == 1) {
+        S.tx[r] = fma(hb, fma(2.0, S.txb[r], -S.tx[r]), ha * S.tx0[r]);
+        S.tw[r] = fma(hb, fma(2.0, S.twb[r], -S.tw[r]), ha * S.tw0[r]);
+      } else if (mode == 2) {
+        S.tx[r] = S.tx0[r] = S.txb[r];
+        S.tw[r] = S.tw0[r] = S.twb[r];
+      }
     }
     if (tid < m) {
       // Halpern / restart on y (m <= 32: one thread per row)
@@ -474,12 +556,51 @@ __device__ void solve_one(const Pools& P, int idx, Shared<PC>& S) {
     __syncthreads();
     // P2-P3: Q wbar_{1/2} (+ Q xbar), v = what + sigma (Q w - Q wbar_{1/2})
     if (HQ) {
-      if (I.p) dense_fx(fac<FS, PC>(P, I), I.p, n, wh, ttest ? xb : nullptr, S.t0, S.t1);
+      if (I.p) {
+        if (listed) {
+          // list the coordinates of xbar that are not 0 (in order: the sums do not depend on timing)
+          const int nwords = (int)((n + 31) >> 5);
+          if (tid < 32) {
+            int at = 0;
+            for (int w0 = 0; w0 < nwords; w0 += 32) {
+              const int c = w0 + tid < nwords ? __popc(S.bits[w0 + tid]) : 0;
+              int sum = c;
+#pragma unroll
+              for (int o = 1; o < 32; o <<= 1) {
+                const int u = __shfl_up_sync(0xffffffffu, sum, o);
+                if (tid >= o) sum += u;
+              }
+              if (w0 + tid < nwords) S.first[w0 + tid] = (unsigned short)(at + sum - c);
+              at += __shfl_sync(0xffffffffu, sum, 31);
+            }
+            if (tid == 0) S.nz = at;
+          }
+          __syncthreads();
+        }
+        const int nz = listed ? S.nz : kMaxList + 1;
+        if (nz <= kMaxList && nz * (int64_t)8 <= n) {
+          for (int64_t jb = tid & ~31; jb < n; jb += nt) {
+            const unsigned b = S.bits[jb >> 5];
+            if ((b >> (tid & 31)) & 1u) {
+              const int at = S.first[jb >> 5] + __popc(b & ((1u << (tid & 31)) - 1u));
+              S.idx[at] = (unsigned short)(jb + (tid & 31));
+              S.val[at] = xb[jb + (tid & 31)];
+            }
+          }
+          __syncthreads();
+          sparse_fx(fac<FS, PC>(P, I), I.p, n, S.idx, S.val, nz, S.txb);
+        } else {
+          dense_fx(fac<FS, PC>(P, I), I.p, n, xb, S.txb);
+        }
+        __syncthreads();
+        // F wbar_{1/2} from eq. (3.3): wbar_{1/2} = c2 (2 xbar - x) + c1 w
+        for (int64_t r = tid; r < I.p; r += nt) S.t0[r] = fma(c2, fma(2.0, S.txb[r], -S.tx[r]), c1 * S.tw[r]);
+      }
       __syncthreads();
       for (int64_t j = tid; j < n; j += nt) {
         const double qwh = q_row<FS, PC>(P, I, j, wh, S.t0);
         Qwh[j] = qwh;
-        if (ttest) Qxb[j] = q_row<FS, PC>(P, I, j, xb, S.t1);
+        if (ttest) Qxb[j] = q_row<FS, PC>(P, I, j, xb, S.txb);
         if (m > 0) v[j] = fma(sg, Qw[j] - qwh, v[j]);
       }
       __syncthreads();
@@ -499,7 +620,12 @@ __device__ void solve_one(const Pools& P, int idx, Shared<PC>& S) {
       }
       __syncthreads();
     }
-    // P5: A^* ybar, wbar (eq. (3.3)), Q wbar by linearity, the R~ / eta / theta~ sums
+    // P5: A^* ybar, wbar (eq. (3.3)), Q wbar and F wbar by linearity, the R~ / eta / theta~ sums
+    for (int64_t r = tid; r < I.p; r += nt) {
+      double q = 0.0;
+      for (int64_t i = 0; i < m; i++) q = fma(fat[r * m + i], S.yb[i] - S.y[i], q);
+      S.twb[r] = fma(sq, q, S.t0[r]);
+    }
     for (int64_t j = tid; j < n; j += nt) {
       double atyb = 0.0, dq = 0.0;
       if (m > 0) {
@@ -546,60 +672,63 @@ __device__ void solve_one(const Pools& P, int idx, Shared<PC>& S) {
         T[11] += conj_phi_term(I.phi, zb[j], L[j], U[j], I.lambda);
       }
     }
-    if (rtest || ttest) block_reduce<kTerms>(T, kMaxMask, S.red);
+    if (rtest || ttest) block_reduce<kTerms>(T, kMaxMask, S.red, (rtest ? 0x7017u : 0u) | (ttest ? 0xfe0u : 0u));
     __syncthreads();
-    // P6: controller (one thread)
-    if (tid == 0) {
-      double Ls[kWL], P3[kW3];
-#pragma unroll
-      for (int q = 0; q < kWL; q++) Ls[q] = T[q];
-      P3[0] = P3[1] = P3[2] = P3[3] = 0.0;
-      double th3 = 0.0, th3r = 0.0, dyr2 = 0.0;
-      for (int64_t i = 0; i < m; i++) {
-        const double dy = S.y[i] - S.yb[i];
-        const double dr = S.yb[i] - S.y0[i];
-        P3[0] = fma(dy, dy, P3[0]);
-        dyr2 = fma(dr, dr, dyr2);
-        if (ttest) {
-          const double ax = S.ax[i], lo = S.lo[i], hi = S.hi[i], ybv = S.yb[i];
-          P3[1] = fmax(P3[1], fabs(ax - fmin(fmax(ax, lo), hi)));
-          P3[2] = fmax(P3[2], fabs(ax));
-          if (ybv > 0.0) P3[3] += lo * ybv;
-          else if (ybv < 0.0) P3[3] += hi * ybv;
-        }
-        if (HQ) {
-          double qd = 0.0, qr = 0.0;
-          for (int64_t l2 = 0; l2 < m; l2++) {
-            qd = fma(aqa[i * m + l2], S.y[l2] - S.yb[l2], qd);
-            qr = fma(aqa[i * m + l2], S.yb[l2] - S.y0[l2], qr);
+    // P6: the m-row sums and quadratic forms (one lane per row), the controller (one thread), Algorithm 5 (the
+    // warp); a dependent FP64 operation takes 64 cycles, and all other warps wait here
+    if (tid < 32) {
+      double p3[kW3] = {0.0, 0.0, 0.0, 0.0}, th3 = 0.0, th3r = 0.0, dyr2 = 0.0;
+      if (rtest || ttest) {
+        const int i = tid;
+        if (i < m) {
+          const double dy = S.y[i] - S.yb[i], dr = S.yb[i] - S.y0[i];
+          p3[0] = dy * dy;
+          dyr2 = dr * dr;
+          if (ttest) {
+            const double ax = S.ax[i], lo = S.lo[i], hi = S.hi[i], ybv = S.yb[i];
+            p3[1] = fabs(ax - fmin(fmax(ax, lo), hi));
+            p3[2] = fabs(ax);
+            if (ybv > 0.0) p3[3] = lo * ybv;
+            else if (ybv < 0.0) p3[3] = hi * ybv;
           }
-          th3 = fma(dy, qd, th3);
-          th3r = fma(dr, qr, th3r);
+          if (HQ && rtest) {
+            double qd = 0.0, qr = 0.0;
+            for (int64_t l2 = 0; l2 < m; l2++) {
+              qd = fma(aqa[i * m + l2], S.y[l2] - S.yb[l2], qd);
+              qr = fma(aqa[i * m + l2], S.yb[l2] - S.y0[l2], qr);
+            }
+            th3 = dy * qd;
+            th3r = dr * qr;
+          }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+          p3[0] += __shfl_xor_sync(0xffffffffu, p3[0], o);
+          dyr2 += __shfl_xor_sync(0xffffffffu, dyr2, o);
+          th3 += __shfl_xor_sync(0xffffffffu, th3, o);
+          th3r += __shfl_xor_sync(0xffffffffu, th3r, o);
+          if (ttest) {
+            p3[1] = fmax(p3[1], __shfl_xor_sync(0xffffffffu, p3[1], o));
+            p3[2] = fmax(p3[2], __shfl_xor_sync(0xffffffffu, p3[2], o));
+            p3[3] += __shfl_xor_sync(0xffffffffu, p3[3], o);
+          }
         }
       }
-      // the single-instance controller expects s * theta_3 in Ls[3]
-      Ls[3] = C.s * th3;
-      const long long r_before = C.r;
-      controller(C, Ls, P3);
+      if (tid == 0) {
+        double Ls[kWL];
+#pragma unroll
+        for (int q = 0; q < kWL; q++) Ls[q] = T[q];
+        // the single-instance controller expects s * theta_3 in Ls[3]
+        Ls[3] = C.s * th3;
+        controller(C, Ls, p3);
+      }
+      __syncwarp();
       if (C.restart_pending) {
         // Algorithm 5 with theta~ of eq. (3.11) from ubar^{r,tau_r} - u^{r,0}
-        double t1 = C.lamA * dyr2 + C.lamQ * T[13] - 2.0 * T[14];
-        double t2 = T[12];
-        t1 = fmax(t1, 1e-12);
-        t2 = fmax(t2, 1e-12);
-        double snew;
-        sigma_argmin_dev(t1, t2, th3r, C.lamQ, C.sigma_golden, &snew);
-        const double beta = exp(-C.ratio);
-        const double sgn = exp(beta * log(snew) + (1.0 - beta) * log(C.sigma));
-        if (!isfinite(sgn) || !(sgn > 0.0)) {
-          C.status = 3;
-          C.done = 1;
-        } else {
-          set_sigma(C, sgn);
-        }
-        C.restart_pending = 0;
+        const double t12 = __shfl_sync(0xffffffffu, T[12], 0), t13 = __shfl_sync(0xffffffffu, T[13], 0),
+                     t14 = __shfl_sync(0xffffffffu, T[14], 0);
+        algorithm5(C, dyr2, t13, t14, t12, th3r);
       }
-      (void)r_before;
     }
     __syncthreads();
   }
@@ -812,7 +941,7 @@ static hprqp_status batch_create_impl(hprqp_batch* b, int32_t count, const hprqp
   std::vector<double> c, L, U, d, x0in, l, u, y0in, F;
   std::vector<int> arp, aci, trp, tci, qrp, qci;
   std::vector<double> av, tv, qv;
-  int64_t qat_total = 0, aqa_total = 0;
+  int64_t qat_total = 0, aqa_total = 0, fat_total = 0;
   b->hinst.resize(count);
   for (int32_t i = 0; i < count; i++) {
     const hprqp_problem& pr = probs[i];
@@ -974,6 +1103,8 @@ static hprqp_status batch_create_impl(hprqp_batch* b, int32_t count, const hprqp
     qat_total += n * m;
     I.oaqa = aqa_total;
     aqa_total += m * m;
+    I.ofat = fat_total;
+    fat_total += I.p * m;
     b->hinst[i] = I;
     b->n_of.push_back(n);
     b->m_of.push_back(m);
@@ -1065,6 +1196,7 @@ static hprqp_status batch_create_impl(hprqp_batch* b, int32_t count, const hprqp
     if ((st = bzeros(b, p, M))) return st;
   if ((st = bzeros(b, &P.qat, (size_t)qat_total))) return st;
   if ((st = bzeros(b, &P.aqa, (size_t)aqa_total))) return st;
+  if ((st = bzeros(b, &P.fat, (size_t)fat_total))) return st;
   int* ip;
   if ((st = bupload(b, &ip, arp))) return st;
   P.arp = ip;
@@ -1138,6 +1270,13 @@ static bool small_p(const Sched& S, int bk) { return S.pmax[bk] <= kSmallP; }
 static size_t bucket_smem(const Sched& S, int bk, bool fs) {
   return shared_bytes(small_p(S, bk)) + (fs ? (size_t)S.fmax[bk] * sizeof(double) : 0);
 }
+// Large blocks of a launch that would not fill the GPU twice are kept one to an SM by their shared memory
+// (just over half of it): two n = 5000 instances on one SM share its FP64 pipe and end the batch at 0.7 s
+// while other SMs idle, and blocks of the buckets behind still fit beside one.
+static size_t launch_smem(const Sched& S, int bk, bool fs, int cnt, int threads, int sms) {
+  const size_t need = bucket_smem(S, bk, fs);
+  return threads >= 512 && cnt < 2 * sms ? std::max(need, (size_t)116 * 1024) : need;
+}
 
 // One launch: the instances order[beg .. beg + cnt) of bucket bk with the given block size and F
 // copy, at most one wave of resident blocks (each takes instances from the bucket's counter).
@@ -1145,7 +1284,7 @@ static cudaError_t launch_bucket(hprqp_batch* b, int bk, int beg, int cnt, int t
                                  cudaStream_t s) {
   const Sched& S = b->sched;
   const KFn k = batch_kernel(fs, small_p(S, bk));
-  const size_t smem = bucket_smem(S, bk, fs);
+  const size_t smem = launch_smem(S, bk, fs, cnt, threads, sms);
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   int occ = 0;
   if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, threads, smem);
