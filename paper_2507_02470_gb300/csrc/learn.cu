@@ -23,6 +23,7 @@
 
 #include "../../include/hprqp_learn.h"
 #include "tc_gemm.cuh"
+#include "tc_ptx.cuh"
 
 namespace {
 
@@ -248,51 +249,29 @@ __global__ void k_col_mean(const double* __restrict__ Z, int64_t rows, int64_t c
 
 // ------------------------------------------------------------------------ transposing epilogues
 // 32 x 32 tiles through shared memory; block (32, 8).
-enum EpiMode { EPI_HIDDEN = 0, EPI_FINAL = 1, EPI_MASK = 2, EPI_STD = 3 };
 
-// Source: FP32 feature-major acc (R x B, ldacc).
-//   HIDDEN: v = bf16(relu(acc + bias))  -> outT (R x ldT), outB (B x ldB)
-//   FINAL:  Y[b][j] = acc + bias        (FP32 batch-major)
-//   MASK:   v = bf16(acc * [mask > 0])  -> outT, outB   (mask: BF16 feature-major, ldmask)
-//   STD:    v = bf16((acc - bias) * scl) -> outB only   (feature standardisation)
-template <int MODE>
-__global__ void k_epi(const float* __restrict__ acc, int64_t ldacc, int R, int B, const float* __restrict__ bias,
-                      const float* __restrict__ scl, const uint16_t* __restrict__ mask, int64_t ldmask,
-                      uint16_t* __restrict__ outB, int64_t ldB, uint16_t* __restrict__ outT, int64_t ldT,
-                      float* __restrict__ Y, int64_t ldy) {
+// Feature standardisation: outB[b][j] = bf16((acc[j][b] - mean[j]) * istd[j]) of FP32 feature-major acc (R x B, ldacc)
+__global__ void k_standardize(const float* __restrict__ acc, int64_t ldacc, int R, int B, const float* __restrict__ mean,
+                              const float* __restrict__ istd, uint16_t* __restrict__ outB, int64_t ldB) {
   __shared__ float tile[32][33];
   const int j0 = blockIdx.y * 32, b0 = blockIdx.x * 32;
   for (int jj = threadIdx.y; jj < 32; jj += 8) {
     const int j = j0 + jj, b = b0 + threadIdx.x;
     float v = 0.f;
-    if (j < R && b < B) {
-      v = acc[(int64_t)j * ldacc + b];
-      if (MODE == EPI_HIDDEN || MODE == EPI_FINAL) v += bias[j];
-      if (MODE == EPI_HIDDEN) v = fmaxf(v, 0.f);
-      if (MODE == EPI_MASK) v = bf16_to_f(mask[(int64_t)j * ldmask + b]) > 0.f ? v : 0.f;
-      if (MODE == EPI_STD) v = (v - bias[j]) * scl[j];
-      if (MODE != EPI_FINAL) {
-        const uint16_t h = f_to_bf16(v);
-        v = bf16_to_f(h);
-        if (MODE != EPI_STD) outT[(int64_t)j * ldT + b] = h;
-      }
-    }
+    if (j < R && b < B) v = (acc[(int64_t)j * ldacc + b] - mean[j]) * istd[j];
     tile[jj][threadIdx.x] = v;
   }
   __syncthreads();
   for (int bb = threadIdx.y; bb < 32; bb += 8) {
     const int b = b0 + bb, j = j0 + threadIdx.x;
-    if (b < B && j < R) {
-      const float v = tile[threadIdx.x][bb];
-      if (MODE == EPI_FINAL) Y[(int64_t)b * ldy + j] = v;
-      else outB[(int64_t)b * ldB + j] = f_to_bf16(v);
-    }
+    if (b < B && j < R) outB[(int64_t)b * ldB + j] = f_to_bf16(tile[threadIdx.x][bb]);
   }
 }
 
 // Source: batch-major FP32 (B x R, ld) -> BF16 batch-major outB and feature-major outT
 __global__ void k_from_batch_f32(const float* __restrict__ src, int64_t ld, int R, int B, uint16_t* __restrict__ outB,
                                  int64_t ldB, uint16_t* __restrict__ outT, int64_t ldT) {
+  hprqp::tc::pdl_wait();
   __shared__ uint16_t tile[32][34];
   const int j0 = blockIdx.x * 32, b0 = blockIdx.y * 32;
   for (int bb = threadIdx.y; bb < 32; bb += 8) {
@@ -314,6 +293,7 @@ __global__ void k_from_batch_f32(const float* __restrict__ src, int64_t ld, int 
 // BF16 batch-major (B x R, ld) -> feature-major (R x ldT)
 __global__ void k_transpose_bf16(const uint16_t* __restrict__ src, int64_t ld, int R, int B, uint16_t* __restrict__ outT,
                                  int64_t ldT) {
+  hprqp::tc::pdl_wait();
   __shared__ uint16_t tile[32][34];
   const int j0 = blockIdx.x * 32, b0 = blockIdx.y * 32;
   for (int bb = threadIdx.y; bb < 32; bb += 8) {
@@ -327,65 +307,96 @@ __global__ void k_transpose_bf16(const uint16_t* __restrict__ src, int64_t ld, i
   }
 }
 
-// db[j] = sum_b dzT[j][b] (BF16 values, FP64 accumulation in a fixed order)
-__global__ void __launch_bounds__(256) k_rowsum_bf16(const uint16_t* __restrict__ dzT, int64_t ldT, int R, int B,
-                                                     float* __restrict__ db) {
-  __shared__ double red[8];
-  for (int j = blockIdx.x; j < R; j += gridDim.x) {
-    double s = 0.0;
-    for (int b = threadIdx.x; b < B; b += 256) s += (double)bf16_to_f(dzT[(int64_t)j * ldT + b]);
-    const double t = block_sum<256>(s, red);
-    if (threadIdx.x == 0) db[j] = (float)t;
-    __syncthreads();
+// The layers of a network as one launch sees them: kernels that treat every layer alike take them all
+// (a launch per layer and array would cost more than its work: 3 to 5 us each)
+constexpr int kMaxLayers = 16;
+struct LayerSet {
+  int count;
+  int first[kMaxLayers + 1];   // blocks before layer l
+  struct One {
+    float *W, *mW, *vW, *b, *mb, *vb;
+    const float *gW, *gb;
+    uint16_t *Wb, *WbT;
+    const uint16_t* dzT;
+    float* db;
+    int64_t ldw, ldwt, ldT;
+    int dout, din;
+  } l[kMaxLayers];
+  __device__ __forceinline__ int of(int block) const {
+    int k = 0;
+    while (k + 1 < count && block >= first[k + 1]) k++;
+    return k;
   }
+};
+
+// db[j] = sum_b dzT[j][b] (BF16 values, FP64 accumulation in a fixed order), one warp per row of any layer,
+// eight values per load (rows are 16-byte aligned: ldT is a multiple of 8)
+__global__ void __launch_bounds__(256) k_rowsum_bf16(const __grid_constant__ LayerSet set, int B) {
+  hprqp::tc::pdl_wait();
+  const int k = set.of(blockIdx.x), j = (blockIdx.x - set.first[k]) * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  const LayerSet::One& y = set.l[k];
+  if (j >= y.dout) return;
+  const uint16_t* row = y.dzT + (int64_t)j * y.ldT;
+  double s = 0.0;
+  int b = 8 * lane;
+  for (; b + 8 <= B; b += 256) {
+    const uint4 q = *reinterpret_cast<const uint4*>(row + b);
+    const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      s += (double)__uint_as_float(w[i] << 16);
+      s += (double)__uint_as_float(w[i] & 0xffff0000u);
+    }
+  }
+  for (; b < B; b++) {   // a partial group of eight: at most one lane's
+    s += (double)bf16_to_f(row[b]);
+    if ((b & 7) == 7) break;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+  if (lane == 0) y.db[j] = (float)s;
 }
 
-// Adam on a dout x din weight (tiles of 32 x 32, block (32, 8)) refreshing W (BF16, ldw) and
-// W^T (BF16, ldwt); `step` = 0 only refreshes the BF16 copies.
-__global__ void k_adam_w(float* __restrict__ W, float* __restrict__ mW, float* __restrict__ vW,
-                         const float* __restrict__ g, int dout, int din, int step, float lr, float b1, float b2,
-                         float eps, float bc1, float bc2, uint16_t* __restrict__ Wb, int64_t ldw,
-                         uint16_t* __restrict__ WbT, int64_t ldwt) {
+// Adam on every dout x din weight (tiles of 32 x 32, block (32, 8)) refreshing W (BF16, ldw) and
+// W^T (BF16, ldwt), the tiles of column 0 also on the biases of their rows; `step` = 0 only refreshes the
+// BF16 copies.
+__global__ void k_adam(const __grid_constant__ LayerSet set, int step, float lr, float b1, float b2, float eps, float bc1,
+                       float bc2) {
+  hprqp::tc::pdl_wait();
   __shared__ uint16_t tile[32][34];
-  const int i0 = blockIdx.x * 32, j0 = blockIdx.y * 32;   // i: input index (column), j: output row
+  const int k = set.of(blockIdx.x), at = blockIdx.x - set.first[k];
+  const LayerSet::One& y = set.l[k];
+  const int nx = (y.din + 31) / 32;
+  const int i0 = at % nx * 32, j0 = at / nx * 32;   // i: input index (column), j: output row
+  auto adam = [&](float w, float& mm, float& vv, float gi) {
+    const float m = b1 * mm + (1.f - b1) * gi;
+    const float v = b2 * vv + (1.f - b2) * gi * gi;
+    mm = m;
+    vv = v;
+    return w - lr * (m / bc1) / (sqrtf(v / bc2) + eps);
+  };
   for (int jj = threadIdx.y; jj < 32; jj += 8) {
     const int j = j0 + jj, i = i0 + threadIdx.x;
     uint16_t h = 0;
-    if (j < dout && i < din) {
-      const int64_t e = (int64_t)j * din + i;
-      float w = W[e];
+    if (j < y.dout && i < y.din) {
+      const int64_t e = (int64_t)j * y.din + i;
+      float w = y.W[e];
       if (step) {
-        const float gi = g[e];
-        const float m = b1 * mW[e] + (1.f - b1) * gi;
-        const float v = b2 * vW[e] + (1.f - b2) * gi * gi;
-        mW[e] = m;
-        vW[e] = v;
-        w -= lr * (m / bc1) / (sqrtf(v / bc2) + eps);
-        W[e] = w;
+        w = adam(w, y.mW[e], y.vW[e], y.gW[e]);
+        y.W[e] = w;
       }
       h = f_to_bf16(w);
-      Wb[(int64_t)j * ldw + i] = h;
+      y.Wb[(int64_t)j * y.ldw + i] = h;
     }
     tile[jj][threadIdx.x] = h;
   }
   __syncthreads();
   for (int ii = threadIdx.y; ii < 32; ii += 8) {
     const int i = i0 + ii, j = j0 + threadIdx.x;
-    if (i < din && j < dout) WbT[(int64_t)i * ldwt + j] = tile[threadIdx.x][ii];
+    if (i < y.din && j < y.dout) y.WbT[(int64_t)i * y.ldwt + j] = tile[threadIdx.x][ii];
   }
-}
-
-__global__ void k_adam_b(float* __restrict__ b, float* __restrict__ mb, float* __restrict__ vb,
-                         const float* __restrict__ g, int n, float lr, float b1, float b2, float eps, float bc1,
-                         float bc2) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const float gi = g[i];
-  const float m = b1 * mb[i] + (1.f - b1) * gi;
-  const float v = b2 * vb[i] + (1.f - b2) * gi * gi;
-  mb[i] = m;
-  vb[i] = v;
-  b[i] -= lr * (m / bc1) / (sqrtf(v / bc2) + eps);
+  const int j = j0 + threadIdx.x;
+  if (step && i0 == 0 && threadIdx.y == 0 && j < y.dout) y.b[j] = adam(y.b[j], y.mb[j], y.vb[j], y.gb[j]);
 }
 
 // ------------------------------------------------------------------------ warm-start loss
@@ -530,8 +541,7 @@ extern "C" hprqp_status hprqp_ws_standardize(const float* F, int64_t d, int64_t 
   if (!F || !mean || !istd || !X) return lfail(HPRQP_INVALID_ARG, "standardize: null pointer");
   dim3 grid((unsigned)((B + 31) / 32), (unsigned)((d + 31) / 32));
   if (grid.y > 65535) return lfail(HPRQP_INVALID_ARG, "standardize: d too large");
-  k_epi<EPI_STD><<<grid, dim3(32, 8), 0, (cudaStream_t)stream>>>(F, ldf, (int)d, (int)B, mean, istd, nullptr, 0, X,
-                                                                  ldx, nullptr, 0, nullptr, 0);
+  k_standardize<<<grid, dim3(32, 8), 0, (cudaStream_t)stream>>>(F, ldf, (int)d, (int)B, mean, istd, X, ldx);
   LCU(cudaGetLastError());
   return HPRQP_OK;
 }
@@ -554,9 +564,7 @@ struct hprqp_mlp {
   std::vector<MlpLayer> layers;
   std::vector<uint16_t*> actB, actT;  // input of layer l: batch-major (maxB x round8(d_l)), feature-major
   std::vector<uint16_t*> dzB, dzT;    // gradient w.r.t. the output of layer l (before ReLU)
-  float* acc = nullptr;              // FP32 feature-major product (max d x ldT)
-  float* work = nullptr;             // split-K partials
-  int64_t work_floats = 0;
+  int64_t work_floats = 0;           // bound of the K-splits' partial sums (splits x M x N)
   int B = 0;                         // batch of the last forward
   int sms = 148;
   std::vector<void*> allocs;
@@ -626,19 +634,29 @@ extern "C" hprqp_status hprqp_mlp_create(hprqp_mlp** out, int32_t nlayers, const
     }
   }
   n->work_floats = std::max<int64_t>((int64_t)n->sms * 128 * 128, (int64_t)dmax * 8);
-  if ((st = A(&n->acc, (size_t)dmax * n->ldT * 4)) || (st = A(&n->work, (size_t)n->work_floats * 4))) {
-    hprqp_mlp_destroy(n);
-    return st;
-  }
   *out = n;
   return HPRQP_OK;
 }
 
+// Layers [l0, l1) for a joined kernel of blocks(layer) blocks each
+template <class F>
+static LayerSet layer_set(const hprqp_mlp* n, int l0, int l1, F blocks) {
+  LayerSet set;
+  set.count = l1 - l0;
+  set.first[0] = 0;
+  for (int l = l0; l < l1; ++l) {
+    const MlpLayer& y = n->layers[l];
+    set.l[l - l0] = LayerSet::One{y.W, y.mW, y.vW, y.b, y.mb, y.vb, y.gW, y.gb, y.Wb, y.WbT, n->dzT[l], y.gb,
+                                  y.ldw, y.ldwt, n->ldT, y.dout, y.din};
+    set.first[l - l0 + 1] = set.first[l - l0] + blocks(y);
+  }
+  return set;
+}
+static int adam_tiles(const MlpLayer& y) { return ((y.din + 31) / 32) * ((y.dout + 31) / 32); }
+
 static hprqp_status refresh_bf16(hprqp_mlp* n, int l) {
-  MlpLayer& y = n->layers[l];
-  dim3 grid((unsigned)((y.din + 31) / 32), (unsigned)((y.dout + 31) / 32));
-  k_adam_w<<<grid, dim3(32, 8), 0, n->s>>>(y.W, y.mW, y.vW, y.gW, y.dout, y.din, 0, 0.f, 0.f, 0.f, 0.f, 1.f, 1.f, y.Wb,
-                                            y.ldw, y.WbT, y.ldwt);
+  const LayerSet set = layer_set(n, l, l + 1, adam_tiles);
+  k_adam<<<set.first[1], dim3(32, 8), 0, n->s>>>(set, 0, 0.f, 0.f, 0.f, 0.f, 1.f, 1.f);
   LCU(cudaGetLastError());
   return HPRQP_OK;
 }
@@ -677,10 +695,16 @@ extern "C" hprqp_status hprqp_mlp_get_grad(hprqp_mlp* n, int32_t l, float* dW, f
   return HPRQP_OK;
 }
 
+// A layer's product and what follows it (tc_gemm.cuh): one launch, the K-splits of a tile one cluster.
 static hprqp_status mlp_gemm(hprqp_mlp* n, int64_t M, int64_t N, int64_t K, const uint16_t* A, int64_t lda,
-                             const uint16_t* B, int64_t ldb, float* C, int64_t ldc) {
-  const int sp = pick_splits(M, N, K, n->work_floats, n->sms);
-  return gemm(M, N, K, A, lda, B, ldb, C, ldc, sp, n->work, n->s);
+                             const uint16_t* B, int64_t ldb, const hprqp::tc::Layer& l) {
+  // the splits that fill the GPU, at most a cluster's
+  const int sp = std::min(pick_splits(M, N, K, n->work_floats, n->sms), hprqp::tc::kLayerSplits);
+  const char* why = nullptr;
+  const cudaError_t e = hprqp::tc::gemm_layer(M, N, K, A, lda, B, ldb, sp, l, n->s, &why);
+  if (e == cudaErrorInvalidValue && why) return lfail(HPRQP_INVALID_ARG, "gemm: %s", why);
+  if (e != cudaSuccess) return lfail(HPRQP_CUDA_ERROR, "gemm: %s", cudaGetErrorString(e));
+  return HPRQP_OK;
 }
 
 extern "C" hprqp_status hprqp_mlp_forward(hprqp_mlp* n, const uint16_t* X, int64_t ldx, int32_t batch, float* Y,
@@ -695,24 +719,26 @@ extern "C" hprqp_status hprqp_mlp_forward(hprqp_mlp* n, const uint16_t* X, int64
   {
     const int d0 = n->dims[0];
     dim3 grid((unsigned)((d0 + 31) / 32), (unsigned)((B + 31) / 32));
-    k_transpose_bf16<<<grid, dim3(32, 8), 0, n->s>>>(X, ldx, d0, B, n->actT[0], n->ldT);
-    LCU(cudaGetLastError());
+    LCU(hprqp::tc::launch_kernel(true, 1, k_transpose_bf16, grid, dim3(32, 8), 0, n->s, X, ldx, d0, B, n->actT[0], n->ldT));
   }
   for (int l = 0; l < n->L; ++l) {
     MlpLayer& y = n->layers[l];
     const uint16_t* in = l == 0 ? X : n->actB[l];
     const int64_t ldin = l == 0 ? ldx : round8(y.din);
-    if ((st = mlp_gemm(n, y.dout, B, y.din, y.Wb, y.ldw, in, ldin, n->acc, n->ldT))) return st;
-    dim3 grid((unsigned)((B + 31) / 32), (unsigned)((y.dout + 31) / 32));
+    hprqp::tc::Layer e;
+    e.bias = y.b;
     if (l + 1 < n->L) {
-      k_epi<EPI_HIDDEN><<<grid, dim3(32, 8), 0, n->s>>>(n->acc, n->ldT, y.dout, B, y.b, nullptr, nullptr, 0,
-                                                          n->actB[l + 1], round8(y.dout), n->actT[l + 1], n->ldT,
-                                                          nullptr, 0);
+      e.mode = hprqp::tc::LAYER_HIDDEN;
+      e.outB = n->actB[l + 1];
+      e.ldB = round8(y.dout);
+      e.outT = n->actT[l + 1];
+      e.ldT = n->ldT;
     } else {
-      k_epi<EPI_FINAL><<<grid, dim3(32, 8), 0, n->s>>>(n->acc, n->ldT, y.dout, B, y.b, nullptr, nullptr, 0, nullptr, 0,
-                                                         nullptr, 0, Y, ldy);
+      e.mode = hprqp::tc::LAYER_FINAL;
+      e.out = Y;
+      e.ldo = ldy;
     }
-    LCU(cudaGetLastError());
+    if ((st = mlp_gemm(n, y.dout, B, y.din, y.Wb, y.ldw, in, ldin, e))) return st;
   }
   return HPRQP_OK;
 }
@@ -727,24 +753,30 @@ extern "C" hprqp_status hprqp_mlp_backward(hprqp_mlp* n, const float* dY, int64_
   {
     const int dL = n->dims[n->L];
     dim3 grid((unsigned)((dL + 31) / 32), (unsigned)((B + 31) / 32));
-    k_from_batch_f32<<<grid, dim3(32, 8), 0, n->s>>>(dY, lddy, dL, B, n->dzB[n->L - 1], round8(dL), n->dzT[n->L - 1],
-                                                     n->ldT);
-    LCU(cudaGetLastError());
+    LCU(hprqp::tc::launch_kernel(true, 1, k_from_batch_f32, grid, dim3(32, 8), 0, n->s, dY, lddy, dL, B, n->dzB[n->L - 1],
+                                 round8(dL), n->dzT[n->L - 1], n->ldT));
   }
   for (int l = n->L - 1; l >= 0; --l) {
     MlpLayer& y = n->layers[l];
     // dW = dZ^T X   (dout x din), K = batch
-    if ((st = mlp_gemm(n, y.dout, y.din, B, n->dzT[l], n->ldT, n->actT[l], n->ldT, y.gW, y.din))) return st;
-    k_rowsum_bf16<<<(int)std::min(y.dout, 65535), 256, 0, n->s>>>(n->dzT[l], n->ldT, y.dout, B, y.gb);
-    LCU(cudaGetLastError());
+    hprqp::tc::Layer g;
+    g.out = y.gW;
+    g.ldo = y.din;
+    if ((st = mlp_gemm(n, y.dout, y.din, B, n->dzT[l], n->ldT, n->actT[l], n->ldT, g))) return st;
     if (l == 0) break;
     // dX^T = W^T dZ^T  (din x B), masked by the ReLU of the layer below
-    if ((st = mlp_gemm(n, y.din, B, y.dout, y.WbT, y.ldwt, n->dzB[l], round8(y.dout), n->acc, n->ldT))) return st;
-    dim3 grid((unsigned)((B + 31) / 32), (unsigned)((y.din + 31) / 32));
-    k_epi<EPI_MASK><<<grid, dim3(32, 8), 0, n->s>>>(n->acc, n->ldT, y.din, B, nullptr, nullptr, n->actT[l], n->ldT,
-                                                      n->dzB[l - 1], round8(y.din), n->dzT[l - 1], n->ldT, nullptr, 0);
-    LCU(cudaGetLastError());
+    hprqp::tc::Layer e;
+    e.mode = hprqp::tc::LAYER_MASK;
+    e.mask = n->actT[l];
+    e.ldmask = n->ldT;
+    e.outB = n->dzB[l - 1];
+    e.ldB = round8(y.din);
+    e.outT = n->dzT[l - 1];
+    e.ldT = n->ldT;
+    if ((st = mlp_gemm(n, y.din, B, y.dout, y.WbT, y.ldwt, n->dzB[l], round8(y.dout), e))) return st;
   }
+  const LayerSet set = layer_set(n, 0, n->L, [](const MlpLayer& y) { return (y.dout + 7) / 8; });
+  LCU(hprqp::tc::launch_kernel(true, 1, k_rowsum_bf16, dim3(set.first[n->L]), dim3(256), 0, n->s, set, B));
   return HPRQP_OK;
 }
 
@@ -753,14 +785,9 @@ extern "C" hprqp_status hprqp_mlp_adam(hprqp_mlp* n, float lr, float beta1, floa
     return lfail(HPRQP_INVALID_ARG, "mlp_adam: bad arguments");
   const float bc1 = (float)(1.0 - std::pow((double)beta1, (double)t));
   const float bc2 = (float)(1.0 - std::pow((double)beta2, (double)t));
-  for (int l = 0; l < n->L; ++l) {
-    MlpLayer& y = n->layers[l];
-    dim3 grid((unsigned)((y.din + 31) / 32), (unsigned)((y.dout + 31) / 32));
-    k_adam_w<<<grid, dim3(32, 8), 0, n->s>>>(y.W, y.mW, y.vW, y.gW, y.dout, y.din, 1, lr, beta1, beta2, eps, bc1, bc2,
-                                              y.Wb, y.ldw, y.WbT, y.ldwt);
-    k_adam_b<<<(y.dout + 255) / 256, 256, 0, n->s>>>(y.b, y.mb, y.vb, y.gb, y.dout, lr, beta1, beta2, eps, bc1, bc2);
-    LCU(cudaGetLastError());
-  }
+  const LayerSet set = layer_set(n, 0, n->L, adam_tiles);
+  LCU(hprqp::tc::launch_kernel(true, 1, k_adam, dim3(set.first[n->L]), dim3(32, 8), 0, n->s, set, 1, lr, beta1, beta2, eps,
+                               bc1, bc2));
   return HPRQP_OK;
 }
 

@@ -16,11 +16,13 @@
 // left waiting, frees its TMEM and returns.
 #include <cuda.h>
 #include <cudaTypedefs.h>
+#include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
 #include <cstdint>
 #include <mutex>
+#include <type_traits>
 
 #include "tc_gemm.cuh"
 #include "tc_ptx.cuh"
@@ -247,6 +249,210 @@ PFN_cuTensorMapEncodeTiled_v12000 encoder(cudaError_t* err) {
   return fn;
 }
 
+
+// ------------------------------------------------------------------------------------ products of the network
+// A layer's product with everything that follows it, in one launch: the S K-splits of a 128 x BN tile
+// are one thread-block cluster.  Each CTA leaves its FP32 partial tile in its own shared memory (the ring
+// is free by then); after a cluster barrier CTA z adds rows [z R, (z + 1) R) of all S partials, read through
+// distributed shared memory in split order (the sums of k_splitk_sum, bit for bit), and applies the
+// epilogue.  The layers' products are 5 to 9 us each and their followers (split sum, bias, ReLU and BF16
+// conversion, transposed copy) as much again in launches: a training step of 512-1024-1024-257 at batch 256
+// took 28 launches and 203 us, with this form, the joined kernels of learn.cu and programmatic dependent
+// launches 12 launches and 131 us (a cluster launch alone costs about 5 us, most of which these hide).
+struct EpiLayer {
+  const float* bias;        // HIDDEN, FINAL: per row
+  const uint16_t* mask;     // MASK: BF16, M x N, ldmask
+  int64_t ldmask;
+  uint16_t* outT;           // HIDDEN, MASK: BF16, M x N, ldT
+  int64_t ldT;
+  uint16_t* outB;           // ... and transposed, N x M, ldB
+  int64_t ldB;
+  float* out;               // FINAL: transposed, N x M, ldo; PLAIN: M x N, ldo
+  int64_t ldo;
+};
+
+__device__ __forceinline__ uint32_t cluster_rank_addr(uint32_t addr, uint32_t rank) {
+  uint32_t to;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(to) : "r"(addr), "r"(rank));
+  return to;
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+}
+
+template <int BN, int MODE>
+__global__ void __launch_bounds__(128, 1)
+    k_gemm_layer(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb, const EpiLayer e, int M,
+                 int N, int kb_total, int kb_per) {
+  constexpr int kStages = EpiStore::kStages;
+  constexpr int kLd = BN + 4;   // row stride of the partial tile: float4 stores of 8 neighbouring rows hit all banks
+  constexpr uint32_t kBTile = (uint32_t)BN * kBK * 2;
+  static_assert(kBM * kLd * 4 <= kStages * (kATile + kBTile), "the partial tile takes the place of the ring");
+  __shared__ __align__(8) uint64_t bar_full[kStages];
+  __shared__ __align__(8) uint64_t bar_empty[kStages];
+  __shared__ __align__(8) uint64_t bar_done;
+  __shared__ uint32_t tmem_slot;
+  extern __shared__ uint8_t dsm[];
+  const uint32_t base = (smem_u32(dsm) + 1023u) & ~1023u;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int m0 = blockIdx.x * kBM, n0 = blockIdx.y * BN;
+  const int kb0 = blockIdx.z * kb_per;
+  const int nkb = min(kb0 + kb_per, kb_total) - kb0;        // >= 1 (host)
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
+                 "r"((uint32_t)BN)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  if (threadIdx.x == 32) {
+    for (int s = 0; s < kStages; ++s) {
+      mbar_init(smem_u32(&bar_full[s]), 1);
+      mbar_init(smem_u32(&bar_empty[s]), 1);
+    }
+    mbar_init(smem_u32(&bar_done), 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = tmem_slot;
+  pdl_wait();   // the set-up above overlaps the end of the kernel before
+  if (warp == 0 && lane == 0) {
+    for (int i = 0; i < nkb; ++i) {
+      const int s = i % kStages;
+      const uint32_t ph = (uint32_t)(i / kStages) & 1u;
+      if (!mbar_wait(smem_u32(&bar_empty[s]), ph ^ 1u, &g_tc_error, 1)) break;
+      const uint32_t fb = smem_u32(&bar_full[s]);
+      mbar_expect_tx(fb, kATile + kBTile);
+      const int kx = (kb0 + i) * kBK;   // multiple of 64 elements: 16-byte aligned
+      tma_load_2d(base + s * kATile, &ta, fb, kx, m0);
+      tma_load_2d(base + kStages * kATile + s * kBTile, &tb, fb, kx, n0);
+    }
+  } else if (warp == 1 && lane == 0) {
+    constexpr uint32_t idesc = idesc_bf16(kBM, BN);
+    for (int i = 0; i < nkb; ++i) {
+      const int s = i % kStages;
+      const uint32_t ph = (uint32_t)(i / kStages) & 1u;
+      if (!mbar_wait(smem_u32(&bar_full[s]), ph, &g_tc_error, 2)) break;
+      tc_fence_after();
+      const uint64_t ad = sdesc_sw128(base + s * kATile);
+      const uint64_t bd = sdesc_sw128(base + kStages * kATile + s * kBTile);
+#pragma unroll
+      for (int kk = 0; kk < kBK / 16; ++kk)
+        mma_bf16(tmem, ad + 2 * kk, bd + 2 * kk, idesc, (i > 0 || kk > 0) ? 1u : 0u);
+      mma_commit(smem_u32(&bar_empty[s]));
+    }
+    mma_commit(smem_u32(&bar_done));
+  }
+  __syncwarp();
+  const bool ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bar_done), 0, &g_tc_error, 3));
+  tc_fence_after();
+  // every product of this CTA has ended, so no copy or MMA touches the ring any more
+  __syncthreads();
+  float* tile = reinterpret_cast<float*>(dsm + (base - smem_u32(dsm)));
+  if (ok) {
+#pragma unroll 1
+    for (int c0 = 0; c0 < BN; c0 += 32) {
+      uint32_t r[32];
+      tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, r);
+      float4* d = reinterpret_cast<float4*>(tile + (warp * 32 + lane) * kLd + c0);
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        d[j] = make_float4(__uint_as_float(r[4 * j]), __uint_as_float(r[4 * j + 1]), __uint_as_float(r[4 * j + 2]),
+                           __uint_as_float(r[4 * j + 3]));
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 0) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)BN) : "memory");
+  }
+  cluster_sync();
+  // rows of this CTA, in 4 x 4 pieces per thread
+  const int S = (int)gridDim.z, R = ((kBM + S - 1) / S + 3) / 4 * 4;
+  const int r0 = (int)blockIdx.z * R, rows = min(R, kBM - r0);
+  for (int u = threadIdx.x; u < rows / 4 * (BN / 4); u += 128) {
+    const int rr = r0 + u / (BN / 4) * 4, cc = u % (BN / 4) * 4;
+    float v[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) v[i][j] = 0.f;
+    for (int s0 = 0; s0 < S; s0 += 4) {   // four peers' loads in flight, added in split order
+      float4 q[4][4];
+#pragma unroll
+      for (int s = 0; s < 4; ++s) {
+        const uint32_t peer = cluster_rank_addr(smem_u32(tile + rr * kLd + cc), (uint32_t)min(s0 + s, S - 1));
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+                       : "=f"(q[s][i].x), "=f"(q[s][i].y), "=f"(q[s][i].z), "=f"(q[s][i].w)
+                       : "r"(peer + (uint32_t)(i * kLd * 4)));
+      }
+#pragma unroll
+      for (int s = 0; s < 4; ++s)
+        if (s0 + s < S) {
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            v[i][0] += q[s][i].x;
+            v[i][1] += q[s][i].y;
+            v[i][2] += q[s][i].z;
+            v[i][3] += q[s][i].w;
+          }
+        }
+    }
+    const int m = m0 + rr, n = n0 + cc;
+    if (m >= M || n >= N) continue;
+    const int mi = min(4, M - m), ni = min(4, N - n);
+    if constexpr (MODE == LAYER_PLAIN) {
+      for (int i = 0; i < mi; ++i) {
+        float* d = e.out + (int64_t)(m + i) * e.ldo + n;
+        for (int j = 0; j < ni; ++j) d[j] = v[i][j];
+      }
+      continue;
+    }
+    if constexpr (MODE == LAYER_FINAL) {
+      for (int j = 0; j < ni; ++j)
+        for (int i = 0; i < mi; ++i) e.out[(int64_t)(n + j) * e.ldo + m + i] = v[i][j] + e.bias[m + i];
+      continue;
+    }
+    uint16_t h[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const float b = MODE == LAYER_HIDDEN && i < mi ? e.bias[m + i] : 0.f;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        float x = v[i][j];
+        if (MODE == LAYER_HIDDEN) {
+          x = fmaxf(x + b, 0.f);
+        } else {
+          const bool in = i < mi && j < ni;
+          const uint16_t k = in ? e.mask[(int64_t)(m + i) * e.ldmask + n + j] : (uint16_t)0;
+          x = (k & 0x8000u) == 0 && (k & 0x7fffu) != 0 && (k & 0x7fffu) <= 0x7f80u ? x : 0.f;   // mask > 0
+        }
+        h[i][j] = __bfloat16_as_ushort(__float2bfloat16_rn(x));
+      }
+    }
+    // leading dimensions are multiples of 8 and the arrays 256-byte aligned: 8-byte stores of four
+    for (int i = 0; i < mi; ++i) {
+      uint16_t* d = e.outT + (int64_t)(m + i) * e.ldT + n;
+      if (ni == 4) *reinterpret_cast<uint2*>(d) = make_uint2(h[i][0] | (h[i][1] << 16), h[i][2] | (h[i][3] << 16));
+      else
+        for (int j = 0; j < ni; ++j) d[j] = h[i][j];
+    }
+    for (int j = 0; j < ni; ++j) {
+      uint16_t* d = e.outB + (int64_t)(n + j) * e.ldB + m;
+      if (mi == 4) *reinterpret_cast<uint2*>(d) = make_uint2(h[0][j] | (h[1][j] << 16), h[2][j] | (h[3][j] << 16));
+      else
+        for (int i = 0; i < mi; ++i) d[i] = h[i][j];
+    }
+  }
+  cluster_sync();   // no CTA ends while a peer reads its tile
+}
+
 }  // namespace
 
 // 2-D map over a rows x cols BF16 matrix with leading dimension ld; boxes of 64 x box_rows
@@ -279,6 +485,23 @@ cudaError_t launch(const CUtensorMap& ta, const CUtensorMap& tb, const Epi& epi,
   dim3 grid((unsigned)((M + kBM - 1) / kBM), (unsigned)((N + BN - 1) / BN), (unsigned)splits);
   k_gemm_bf16<BN, Epi><<<grid, 128, bytes, s>>>(ta, tb, epi, (int)M, (int)N, kb_total, kb_per);
   return cudaGetLastError();
+}
+
+template <int BN, int MODE>
+cudaError_t launch_layer(const CUtensorMap& ta, const CUtensorMap& tb, const EpiLayer& epi, int64_t M, int64_t N,
+                         int kb_total, int kb_per, int splits, cudaStream_t s) {
+  constexpr uint32_t bytes = smem_bytes<BN, EpiStore::kStages>();
+  static std::once_flag once;
+  static cudaError_t attr = cudaSuccess;
+  std::call_once(once, [] {
+    attr = cudaFuncSetAttribute(k_gemm_layer<BN, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (attr == cudaSuccess)
+      attr = cudaFuncSetAttribute(k_gemm_layer<BN, MODE>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  });
+  if (attr != cudaSuccess) return attr;
+  return launch_kernel(true, splits, k_gemm_layer<BN, MODE>,
+                       dim3((unsigned)((M + kBM - 1) / kBM), (unsigned)((N + BN - 1) / BN), (unsigned)splits), dim3(128),
+                       bytes, s, ta, tb, epi, (int)M, (int)N, kb_total, kb_per);
 }
 
 // The operand checks that every product shares; what is wrong, or null.
@@ -355,6 +578,45 @@ cudaError_t gemm_decode(int64_t D, int64_t N, int64_t K, const void* A, int64_t 
   if ((e = make_map(&tb, B, N, K, ldb, BN)) != cudaSuccess) return e;
   const EpiDecode epi{alpha, mu, lo, hi, Z, ldz};
   return BN == 64 ? launch<64>(ta, tb, epi, D, N, kb, kb, 1, stream) : launch<128>(ta, tb, epi, D, N, kb, kb, 1, stream);
+}
+
+int layer_splits(int64_t K, int splits) {
+  const int kb_total = (int)((K + kBK - 1) / kBK);
+  splits = std::max(1, std::min(splits, kb_total));
+  const int kb_per = (kb_total + splits - 1) / splits;
+  return (kb_total + kb_per - 1) / kb_per;
+}
+
+cudaError_t gemm_layer(int64_t M, int64_t N, int64_t K, const void* A, int64_t lda, const void* B, int64_t ldb,
+                       int splits, const Layer& l, cudaStream_t stream, const char** why) {
+  auto bad = [why](const char* w) {
+    if (why) *why = w;
+    return cudaErrorInvalidValue;
+  };
+  if (M < 1 || N < 1 || K < 1 || M >= (1ll << 31) || N > 65535ll * 64 || K >= (1ll << 31)) return bad("size out of range");
+  if (const char* w = check_operands(M, N, K, A, lda, B, ldb)) return bad(w);
+  const int kb_total = (int)((K + kBK - 1) / kBK);
+  splits = layer_splits(K, splits);
+  if (splits > kLayerSplits) return bad("too many splits for a cluster");
+  const int kb_per = (kb_total + splits - 1) / splits;
+  const int BN = N <= 64 ? 64 : N < 512 ? 128 : 256;   // the tile rule of gemm_bf16
+  CUtensorMap ta, tb;
+  cudaError_t e;
+  if ((e = make_map(&ta, A, M, K, lda, kBM)) != cudaSuccess) return e;
+  if ((e = make_map(&tb, B, N, K, ldb, BN)) != cudaSuccess) return e;
+  const EpiLayer epi{l.bias, l.mask, l.ldmask, l.outT, l.ldT, l.outB, l.ldB, l.out, l.ldo};
+  auto go = [&](auto mode) {
+    constexpr int m = decltype(mode)::value;
+    return BN == 64    ? launch_layer<64, m>(ta, tb, epi, M, N, kb_total, kb_per, splits, stream)
+           : BN == 128 ? launch_layer<128, m>(ta, tb, epi, M, N, kb_total, kb_per, splits, stream)
+                       : launch_layer<256, m>(ta, tb, epi, M, N, kb_total, kb_per, splits, stream);
+  };
+  switch (l.mode) {
+    case LAYER_HIDDEN: return go(std::integral_constant<int, LAYER_HIDDEN>());
+    case LAYER_MASK: return go(std::integral_constant<int, LAYER_MASK>());
+    case LAYER_FINAL: return go(std::integral_constant<int, LAYER_FINAL>());
+    default: return go(std::integral_constant<int, LAYER_PLAIN>());
+  }
 }
 
 int gemm_error_flag() {

@@ -26,6 +26,30 @@ cudaError_t gemm_decode(int64_t D, int64_t N, int64_t K, const void* A, int64_t 
                         double alpha, const double* mu, const double* lo, const double* hi, double* Z, int64_t ldz,
                         cudaStream_t stream, const char** why);
 
+// What follows a layer's product acc (M features x N members), in the same launch:
+//   HIDDEN  v = bf16(relu(acc + bias)) -> outT (M x ldT) and outB (N x ldB)
+//   MASK    v = bf16(acc where mask > 0, else 0) -> outT, outB   (mask: BF16, M x ldmask)
+//   FINAL   out[n][m] = acc + bias (N x ldo)
+//   PLAIN   out[m][n] = acc (M x ldo)
+// outT and outB rows are 8-byte aligned.
+enum LayerMode { LAYER_HIDDEN = 0, LAYER_MASK = 1, LAYER_FINAL = 2, LAYER_PLAIN = 3 };
+struct Layer {
+  int mode = LAYER_PLAIN;
+  const float* bias = nullptr;
+  const uint16_t* mask = nullptr;
+  int64_t ldmask = 0;
+  uint16_t* outT = nullptr;
+  int64_t ldT = 0;
+  uint16_t* outB = nullptr;
+  int64_t ldB = 0;
+  float* out = nullptr;
+  int64_t ldo = 0;
+};
+constexpr int kLayerSplits = 16;              // K-splits of a tile: CTAs of one cluster
+int layer_splits(int64_t K, int splits);      // the splits that a request for `splits` comes to
+cudaError_t gemm_layer(int64_t M, int64_t N, int64_t K, const void* A, int64_t lda, const void* B, int64_t ldb,
+                       int splits, const Layer& l, cudaStream_t stream, const char** why);
+
 // Reads and clears the device flag that a GEMM kernel sets when one of its bounded waits
 // gave up (0: none; 1 producer, 2 MMA issuer, 3 epilogue).  Synchronises the device.
 int gemm_error_flag();

@@ -102,6 +102,39 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
+// Entry of a kernel that may start as a programmatic dependent launch: wait until the kernel before it has
+// ended and its writes are visible (a no-op after an ordinary launch), after letting the next one begin to launch.
+__device__ __forceinline__ void pdl_wait() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// Launches k, with pdl as a programmatic dependent launch (k calls pdl_wait first), with cz > 1 in clusters of
+// cz blocks along z.  Only directly after another kernel on s that has waited for its own predecessor.
+template <typename... P, typename... A>
+cudaError_t launch_kernel(bool pdl, int cz, void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                          A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[2];
+  int n = 0;
+  if (pdl) {
+    at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[n++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (cz > 1) {
+    at[n].id = cudaLaunchAttributeClusterDimension;
+    at[n].val.clusterDim.x = at[n].val.clusterDim.y = 1;
+    at[n++].val.clusterDim.z = (unsigned)cz;
+  }
+  cfg.attrs = at;
+  cfg.numAttrs = (unsigned)n;
+  return cudaLaunchKernelEx(&cfg, k, static_cast<P>(args)...);
+}
+
 // 2-D tensor map over a rows x cols BF16 matrix with leading dimension ld (elements), boxes of 64 columns x
 // box_rows rows, 128-byte swizzle, zeros past the edges (tc_gemm.cu)
 cudaError_t make_map(CUtensorMap* map, const void* ptr, int64_t rows, int64_t cols, int64_t ld, int box_rows);
