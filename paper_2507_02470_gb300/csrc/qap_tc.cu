@@ -23,7 +23,7 @@
 // tile of one product and one or several chunks of 64 k's; a chunk's digits of both operands (172 KB) are
 // fetched with 14 TMA loads behind one mbarrier and multiplied by 136 tcgen05.mma.
 // us per product before a pass, FP64 contractions (qap.cu) / this path: d = 9: 49 / 43, 32: 85 / 43, 64: 162 / 49,
-// 128: 186 / 53, 256: 189 / 62, 400: 728 / 175; at d = 256 the two k_fix take 13 us each.  Below d = 8 one
+// 128: 186 / 53, 256: 189 / 57, 400: 728 / 175; at d = 256 the two k_fix take 13 us each.  Below d = 8 one
 // FP64 tile is as fast.
 #include <algorithm>
 #include <vector>
@@ -139,6 +139,7 @@ __global__ void __launch_bounds__(256) k_slice_rows(const double* src, int d, in
 
 // digits of X by rows (the first blocks, eight rows each) and by columns (32 each)
 __global__ void __launch_bounds__(kFarThreads) k_slice_x(const double* x, QapTcDev q) {
+  tc::pdl_wait();
   const int half = (q.d + 7) / 8;
   if ((int)blockIdx.x < half)
     slice_far([&](int i, int k) { return x[(size_t)k * q.d + i]; }, (int)blockIdx.x * 8, q.d, q.kp, q.plane, q.dig[kXRow],
@@ -165,6 +166,7 @@ __device__ __forceinline__ double join(const QapTcDev& q, int prod, int a, int b
 
 // T1 = Ahat X (kept in t1, column-major) and its digits by rows
 __global__ void __launch_bounds__(kFarThreads) k_slice_t1(QapTcDev q) {
+  tc::pdl_wait();
   const int r0 = blockIdx.x * 8, i = threadIdx.x & 7, g = threadIdx.x >> 3;
   if (r0 + i < q.d)
     for (int k = g; k < q.d; k += 128) q.t1[(size_t)k * q.d + r0 + i] = join(q, 0, kAhat, kXCol, r0 + i, k);
@@ -174,6 +176,7 @@ __global__ void __launch_bounds__(kFarThreads) k_slice_t1(QapTcDev q) {
 
 // out = T1 Bhat - S X - X T
 __global__ void __launch_bounds__(256) k_join(QapTcDev q, double* out) {
+  tc::pdl_wait();
   const int64_t e = (int64_t)blockIdx.x * 256 + threadIdx.x;
   if (e >= (int64_t)q.d * q.d) return;
   const int i = (int)(e % q.d), j = (int)(e / q.d);
@@ -211,6 +214,7 @@ __global__ void __launch_bounds__(128, 1) k_fix(const __grid_constant__ Maps map
   __syncthreads();
   tc::tc_fence_after();
   const uint32_t tmem = tmem_slot;
+  tc::pdl_wait();   // the set-up above overlaps the end of the kernel before
   const size_t dd = (size_t)q.d * q.d;
   long long* part = q.part + ((size_t)(first + prod) * q.groups + group) * 2 * dd;
   bool ok = true;
@@ -250,28 +254,25 @@ __global__ void __launch_bounds__(128, 1) k_fix(const __grid_constant__ Maps map
       const int i = m0 + warp * 32 + lane;
 #pragma unroll 1
       for (int c0 = 0; c0 < kBN; c0 += 32) {
-        long long hi[32], lo[32];
+        // (loops over the sums that are not unrolled: the code is run once, and fetching it would bound it)
+#pragma unroll 1
+        for (int half = 0; half < 2; half++) {
+          long long v[32];
 #pragma unroll
-        for (int s = 0; s < kSum; s++) {
-          uint32_t r[32];
-          tc::tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(s * kBN + c0), r);
+          for (int j = 0; j < 32; j++) v[j] = 0;
+#pragma unroll 1
+          for (int s = half * 4; s < half * 4 + 4; s++) {
+            uint32_t r[32];
+            tc::tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(s * kBN + c0), r);
 #pragma unroll
-          for (int j = 0; j < 32; j++) {
-            const long long v = (long long)__float2int_rn(__uint_as_float(r[j]));
-            if (s == 0) hi[j] = v;
-            else if (s < 4) hi[j] = hi[j] * 256 + v;
-            else if (s == 4) lo[j] = v;
-            else lo[j] = lo[j] * 256 + v;
+            for (int j = 0; j < 32; j++) v[j] = v[j] * 256 + (long long)__float2int_rn(__uint_as_float(r[j]));
           }
-        }
-        if (i < q.d) {
+          if (i < q.d) {
+            long long* h = part + (half ? dd : 0) + (size_t)(n0 + c0) * q.d + i;
 #pragma unroll
-          for (int j = 0; j < 32; j++)
-            if (n0 + c0 + j < q.d) {
-              long long* h = part + (size_t)(n0 + c0 + j) * q.d + i;
-              h[0] = it ? h[0] + hi[j] : hi[j];
-              h[dd] = it ? h[dd] + lo[j] : lo[j];
-            }
+            for (int j = 0; j < 32; j++, h += q.d)
+              if (n0 + c0 + j < q.d) *h = it ? *h + v[j] : v[j];
+          }
         }
       }
     }
@@ -357,15 +358,17 @@ cudaError_t qap_tc_create(QapTc** out, int64_t d, const double* mats, void* mem,
   return cudaSuccess;
 }
 
-cudaError_t qap_tc_apply(const QapTc* t, const double* x, double* out, cudaStream_t s) {
+cudaError_t qap_tc_apply(const QapTc* t, const double* x, double* out, bool pdl, cudaStream_t s) {
   const QapTcDev& q = t->dev;
   const int rows = (q.d + 7) / 8, tiles = ((q.d + kBM - 1) / kBM) * ((q.d + kBN - 1) / kBN);
-  k_slice_x<<<rows + (q.d + 31) / 32, kFarThreads, 0, s>>>(x, q);
-  k_fix<<<3 * tiles * q.groups, 128, kFixSmem, s>>>(t->one, q, 0);
-  k_slice_t1<<<rows, kFarThreads, 0, s>>>(q);
-  k_fix<<<tiles * q.groups, 128, kFixSmem, s>>>(t->two, q, 3);
-  k_join<<<(int)(((int64_t)q.d * q.d + 255) / 256), 256, 0, s>>>(q, out);
-  return cudaGetLastError();
+  const dim3 far(kFarThreads), fix(128), flat(256);
+  cudaError_t e = tc::launch_kernel(false, 1, k_slice_x, dim3(rows + (q.d + 31) / 32), far, 0, s, x, q);
+  if (e == cudaSuccess) e = tc::launch_kernel(pdl, 1, k_fix, dim3(3 * tiles * q.groups), fix, kFixSmem, s, t->one, q, 0);
+  if (e == cudaSuccess) e = tc::launch_kernel(pdl, 1, k_slice_t1, dim3(rows), far, 0, s, q);
+  if (e == cudaSuccess) e = tc::launch_kernel(pdl, 1, k_fix, dim3(tiles * q.groups), fix, kFixSmem, s, t->two, q, 3);
+  if (e == cudaSuccess)
+    e = tc::launch_kernel(pdl, 1, k_join, dim3((unsigned)(((int64_t)q.d * q.d + 255) / 256)), flat, 0, s, q, out);
+  return e;
 }
 
 }  // namespace hprqp

@@ -26,8 +26,8 @@ size_t qap_tc_bytes(int64_t d, size_t (&part)[5]);
 cudaError_t qap_tc_create(QapTc** out, int64_t d, const double* mats, void* mem, cudaStream_t s);
 void qap_tc_free(QapTc* t);
 const int* qap_tc_error(const QapTc* t);   // device word
-// out = vec(Ahat X Bhat - S X - X T): five kernels
-cudaError_t qap_tc_apply(const QapTc* t, const double* x, double* out, cudaStream_t s);
+// out = vec(Ahat X Bhat - S X - X T): five kernels; pdl: the last four as programmatic dependent launches
+cudaError_t qap_tc_apply(const QapTc* t, const double* x, double* out, bool pdl, cudaStream_t s);
 constexpr int kQapTcKernels = 5;
 
 }  // namespace hprqp

@@ -88,7 +88,7 @@ cudaError_t launch_qap(const Args& a, const Plan& p, int which, int tt, cudaStre
     if (e != cudaSuccess) return e;
   }
   auto apply = [&](const double* v, double* out) {
-    return Q.qap_tc ? qap_tc_apply(Q.qap_tc, v, out, s) : qap_apply(Q, v, out, Q.qap_splits, s);
+    return Q.qap_tc ? qap_tc_apply(Q.qap_tc, v, out, p.pdl != 0, s) : qap_apply(Q, v, out, Q.qap_splits, s);
   };
   cudaError_t e = apply(x, t + Q.qap_off);
   if (e == cudaSuccess && which == 0 && tt != 0) e = apply(V.xb, t + Q.tlen + Q.qap_off);
@@ -185,6 +185,7 @@ cudaError_t launch_step(const Args& a, const Plan& p, cudaStream_t s, int var, c
       L.other();
       const cudaError_t qe = launch_qap(a, p, which, ptt, s);
       if (qe != cudaSuccess) return qe;
+      if (a.Q.qap_tc) L.prev = true;   // its last kernel has waited for its predecessors
       L.count += qap_kernels(a) * (which == PRE_WH && ptt != 0 ? 2 : 1);
     }
     return cudaSuccess;
