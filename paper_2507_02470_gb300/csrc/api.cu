@@ -952,10 +952,6 @@ static hprqp_status create_impl(hprqp_handle* h, int64_t n, int64_t m, const hpr
   if (m > 0) {
     if ((st = upload_csr(h, a.A, A))) return st;
     if ((st = upload_transpose(h, a.AT, a.A, A))) return st;
-    // SELL copies for the autotuner's choice (not for the persistent mode, which keeps lanes)
-    if (h->prm.launch_mode != 3 && h->prm.autotune != 0) {
-      if ((st = build_sell_rows(h, a.A)) || (st = build_sell_rows(h, a.AT))) return st;
-    }
   } else {
     a.A.cols = n;
     a.AT.cols = 0;
@@ -1213,8 +1209,28 @@ static hprqp_status create_impl(hprqp_handle* h, int64_t n, int64_t m, const hpr
   CU(h, cudaStreamSynchronize(h->stream));
 
   clk.mark("launch plan");
-  // ---- schedule autotune (lanes per row for each CSR pass)
-  {
+  if ((st = plan_resident(h, A, qcsr, thin, facs, sms))) return st;
+  clk.mark("resident plan");
+  // ---- schedule of the separate kernels (lanes per row for each CSR pass)
+  if (h->res.B) {
+    // solves run resident: the separate kernels (hprqp_apply, hprqp_profile) take the lanes that the mean row
+    // length suggests, and the probes (2 ms, a quarter of a small problem's create) are left out
+    const int tune = h->prm.autotune;
+    h->prm.autotune = 0;
+    P.gA = m > 0 ? tune_G(h, a.A, a.rowsA, P.gridM, ain, aout, 1) : 1;
+    P.gAT = m > 0 ? tune_G(h, a.AT, kChunk, P.gridN, ain, aout, 1) : 1;
+    const Csr* big = QD.csr.rows ? &QD.csr : nullptr;
+    for (int f = 0; f < QD.nfac; f++)
+      if (!QD.inl[f] && (!big || QD.fact[f].nnz > big->nnz)) big = &QD.fact[f];
+    P.gQ = big ? tune_G(h, *big, kChunk, P.gridN, ain, aout, 1) : 1;
+    h->prm.autotune = tune;
+    CU(h, plan_plain_grids(a, P, sms));
+    P.fuse = m > 0 ? 1 : 0;
+  } else {
+    // SELL copies for the autotuner's choice (not for the persistent mode, which keeps lanes)
+    if (m > 0 && h->prm.launch_mode != 3 && h->prm.autotune != 0) {
+      if ((st = build_sell_rows(h, a.A)) || (st = build_sell_rows(h, a.AT))) return st;
+    }
     CU(h, cudaMemsetAsync(ain, 0, nm * sizeof(double), h->stream));
     P.gA = m > 0 ? tune_G(h, a.A, a.rowsA, P.gridM, ain, aout, 1) : 1;
     P.gAT = m > 0 ? tune_G(h, a.AT, kChunk, P.gridN, ain, aout, 1) : 1;
@@ -1259,7 +1275,6 @@ static hprqp_status create_impl(hprqp_handle* h, int64_t n, int64_t m, const hpr
     // plain steps of the fixed-schedule graph end with the fused passes (need Q and A)
     P.fuse = (h->prm.fused_steps != 0 && QD.present() && m > 0) ? 1 : 0;
   }
-  if ((st = plan_resident(h, A, qcsr, thin, facs, sms))) return st;
   clk.mark("autotune");
   return HPRQP_OK;
 }
