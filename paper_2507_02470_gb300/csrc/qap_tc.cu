@@ -161,7 +161,9 @@ __device__ __forceinline__ double join(const QapTcDev& q, int prod, int a, int b
   }
   const long long hi = (h[0] + h[1]) + (h[2] + h[3]), lo = (l[0] + l[1]) + (l[2] + l[3]);
   // hi < 2^53 and lo < 2^53 are exact in FP64
-  return fma((double)hi, 4294967296.0, (double)lo) * q.scale[a][i] * q.scale[b][j];
+  // the smaller scale first: a product in FP64's range does not overflow on the way to it
+  const double v = fma((double)hi, 4294967296.0, (double)lo), sa = q.scale[a][i], sb = q.scale[b][j];
+  return sa < sb ? v * sa * sb : v * sb * sa;
 }
 
 // T1 = Ahat X (kept in t1, column-major) and its digits by rows
