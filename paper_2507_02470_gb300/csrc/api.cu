@@ -609,12 +609,25 @@ static std::vector<int> column_pointers(const HostCsr& M) {
   return cp;
 }
 
+// row pointers of the thin factors' explicit B^T B (QDev::thin)
+static std::vector<int> thin_pointers(const std::vector<HostCsr>& facs, const QDev& Q, int64_t n) {
+  std::vector<int> rp(n + 1, 0);
+  for (int f = 0; f < Q.nfac; f++) {
+    if (!Q.inl[f]) continue;
+    const HostCsr& B = facs[f];
+    for (int64_t r = 0; r < B.rows; r++)
+      for (int k = B.rp[r]; k < B.rp[r + 1]; k++) rp[B.ci[k] + 1] += B.rp[r + 1] - B.rp[r];
+  }
+  for (int64_t j = 0; j < n; j++) rp[j + 1] += rp[j];
+  return rp;
+}
+
 // Splits the problem over blocks for the resident solver and lays out their shared memory (p.B stays
 // 0 when it does not apply).  It takes what needs no more than the state in shared memory: matrices
 // that do not fit beside it are read through L2.  Options that ask for a schedule of the separate
 // kernels (launch_mode, fixed_schedule, fused_steps, pdl, autotune, factor_inline, tiled_factor other than their
 // defaults) get that schedule.
-static hprqp_status plan_resident(hprqp_handle* h, const HostCsr& A, const HostCsr& qcsr, const HostCsr& thin,
+static hprqp_status plan_resident(hprqp_handle* h, const HostCsr& A, const HostCsr& qcsr,
                                   const std::vector<HostCsr>& facs, int sms) {
   const hprqp_params& q = h->prm;
   const QDev& Q = h->args.Q;
@@ -666,7 +679,7 @@ static hprqp_status plan_resident(hprqp_handle* h, const HostCsr& A, const HostC
   p.gA = lanes(m, annz, p.rm);
   p.gAT = lanes(n, annz, p.rn);
   p.gQ = lanes(n, qnnz, p.rn);
-  p.gT = thin.rp.empty() ? 1 : lanes(n, thin.rp[n], p.rn);
+  p.gT = Q.thin.rows ? lanes(n, Q.thin.nnz, p.rn) : 1;
   p.gF = lanes(n, fnnz, p.rn);
   p.gP = lanes(frows, fnnz, p.rp);
   p.cw = 32;
@@ -701,7 +714,7 @@ static hprqp_status plan_resident(hprqp_handle* h, const HostCsr& A, const HostC
     place(p.AT, most_entries(column_pointers(A), n, p.rn), p.rn);
   }
   if (qcsr.rows) place(p.Qc, most_entries(qcsr.rp, n, p.rn), p.rn);
-  if (!thin.rp.empty()) place(p.thin, most_entries(thin.rp, n, p.rn), p.rn);
+  if (Q.thin.rows) place(p.thin, most_entries(thin_pointers(facs, Q, n), n, p.rn), p.rn);
   for (int f = 0; f < Q.nfac; f++) {
     place(p.fact[f], most_entries(column_pointers(facs[f]), n, p.rn), p.rn);
     if (!Q.inl[f]) place(p.fac[f], most_entries(facs[f].rp, facs[f].rows, p.rp, Q.toff[f]), p.rp);
@@ -1051,10 +1064,10 @@ static hprqp_status create_impl(hprqp_handle* h, int64_t n, int64_t m, const hpr
   // ---- thin factor terms: the inner step multiplies with the explicit entries of B^T B (sum_r len(r)^2 of
   // them); at most n / 2 they cost less than the pre-pass launch and its latency (S of the n = 1e6 CQP: 1e4
   // rows of 3, 9e4 entries)
-  HostCsr thin;
+  // (formed on the device; on the host it took 5 ms at n = 1e6, most of it for the row pointers)
   {
-    thin.rows = thin.cols = n;
-    double pairs = 0.0;   // entries of all thin terms: 32-bit row pointers
+    ThinTerms T;
+    int64_t pairs = 0;   // entries of all thin terms: 32-bit row pointers
     for (int f = 0; f < QD.nfac; f++) {
       if (QD.tiled[f] || h->prm.factor_inline == 0) continue;
       const HostCsr& B = facs[f];
@@ -1064,31 +1077,28 @@ static hprqp_status create_impl(hprqp_handle* h, int64_t n, int64_t m, const hpr
         sq += l * l;
       }
       if (sq > 0.5 * (double)n && h->prm.factor_inline != 2) continue;
-      if (pairs + sq > 1e9) continue;
-      pairs += sq;
+      if ((double)pairs + sq > 1e9) continue;
+      pairs += (int64_t)sq;
       QD.inl[f] = 1;
-      if (thin.rp.empty()) thin.rp.assign(n + 1, 0);
-      for (int64_t r = 0; r < B.rows; r++)
-        for (int k = B.rp[r]; k < B.rp[r + 1]; k++) thin.rp[B.ci[k] + 1] += B.rp[r + 1] - B.rp[r];
+      void* off;
+      if ((st = dalloc(h, &off, (size_t)(QD.fact[f].nnz + 1) * sizeof(int)))) return st;
+      T.B[T.count] = QD.fac[f];
+      T.BT[T.count] = QD.fact[f];
+      T.off[T.count++] = (int*)off;
     }
-    if (!thin.rp.empty()) {
-      for (int64_t j = 0; j < n; j++) thin.rp[j + 1] += thin.rp[j];
-      thin.ci.resize(thin.rp[n]);
-      thin.v.resize(thin.rp[n]);
-      std::vector<int> at(thin.rp.begin(), thin.rp.end() - 1);
-      for (int f = 0; f < QD.nfac; f++) {
-        if (!QD.inl[f]) continue;
-        const HostCsr& B = facs[f];
-        for (int64_t r = 0; r < B.rows; r++)
-          for (int k = B.rp[r]; k < B.rp[r + 1]; k++) {
-            int& q = at[B.ci[k]];
-            for (int i = B.rp[r]; i < B.rp[r + 1]; i++, q++) {
-              thin.ci[q] = B.ci[i];
-              thin.v[q] = B.v[k] * B.v[i];
-            }
-          }
-      }
-      if ((st = upload_csr(h, QD.thin, thin))) return st;
+    if (T.count) {
+      void *rp, *ci, *v, *mx;
+      if ((st = dalloc(h, &rp, (size_t)(n + 1) * sizeof(int))) || (st = dalloc(h, &mx, sizeof(int))) ||
+          (st = dalloc(h, &ci, (size_t)std::max<int64_t>(pairs, 1) * sizeof(int))) ||
+          (st = dalloc(h, &v, (size_t)std::max<int64_t>(pairs, 1) * sizeof(double))))
+        return st;
+      CU(h, thin_layout(T, n, (int*)rp, (int*)mx, h->stream));
+      CU(h, thin_fill(T, n, (const int*)rp, (int*)ci, (double*)v, h->stream));
+      QD.thin.rows = QD.thin.cols = n;
+      QD.thin.nnz = pairs;
+      QD.thin.rp = (const int*)rp;
+      QD.thin.ci = (const int*)ci;
+      QD.thin.v = (const double*)v;
     }
   }
   QD.tlen = toff;
@@ -1209,7 +1219,7 @@ static hprqp_status create_impl(hprqp_handle* h, int64_t n, int64_t m, const hpr
   CU(h, cudaStreamSynchronize(h->stream));
 
   clk.mark("launch plan");
-  if ((st = plan_resident(h, A, qcsr, thin, facs, sms))) return st;
+  if ((st = plan_resident(h, A, qcsr, facs, sms))) return st;
   clk.mark("resident plan");
   // ---- schedule of the separate kernels (lanes per row for each CSR pass)
   if (h->res.B) {

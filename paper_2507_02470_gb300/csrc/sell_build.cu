@@ -208,40 +208,60 @@ __global__ void k_tr_count(const int* __restrict__ ci, int64_t nnz, int* __restr
     atomicAdd(cnt + ci[q] + 1, 1);
 }
 
-// in-place inclusive scan of rp[0..len) (rp[0] = 0) and the largest difference (one block)
-__global__ void k_tr_scan(int* __restrict__ rp, int64_t len, int* __restrict__ maxlen) {
-  __shared__ long long part[kThreads];
-  __shared__ int mx[kThreads];
-  const int t = threadIdx.x;
-  const int64_t per = (len + kThreads - 1) / kThreads;
-  const int64_t b = t * per, e = b + per < len ? b + per : len;
-  long long sum = 0;
-  int m = 0;
-  for (int64_t i = b; i < e; i++) {
-    sum += rp[i];
-    m = rp[i] > m ? rp[i] : m;
-  }
-  part[t] = sum;
-  mx[t] = m;
-  __syncthreads();
-  if (t == 0) {
-    long long run = 0;
-    int mm = 0;
-    for (int i = 0; i < kThreads; i++) {
-      const long long v = part[i];
-      part[i] = run;
-      run += v;
-      mm = mx[i] > mm ? mx[i] : mm;
+// in-place inclusive scan of rp[0..len) (rp[0] = 0) and the largest element (one block of kScanThreads): tiles
+// of kScanThreads * kScanPer elements, read and written coalesced, the carry kept by every thread.  One block
+// because a scan is a small part of a create; bound by the latency of its tiles' loads and barriers.  With
+// each of 256 threads walking its own part of the array (uncoalesced), uploads and transposes of the n = 1e6,
+// m = 5e5 CQP took 5.2 ms of its create, now 2.4.
+constexpr int kScanThreads = 1024, kScanPer = 4;
+__global__ __launch_bounds__(kScanThreads) void k_tr_scan(int* __restrict__ rp, int64_t len,
+                                                          int* __restrict__ maxlen) {
+  __shared__ int warp_sum[2][kScanThreads / 32];
+  __shared__ int warp_max[kScanThreads / 32];
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+  int carry = 0, m = 0, buf = 0;
+  for (int64_t base = 0; base < len; base += kScanThreads * kScanPer, buf ^= 1) {
+    // a warp owns 32 * kScanPer consecutive elements, lane l the elements l, l + 32, ..
+    const int64_t at = base + (int64_t)w * 32 * kScanPer + lane;
+    int x[kScanPer];
+#pragma unroll
+    for (int k = 0; k < kScanPer; k++) x[k] = at + 32 * k < len ? rp[at + 32 * k] : 0;
+    int run = 0;   // sum of the warp's elements so far
+#pragma unroll
+    for (int k = 0; k < kScanPer; k++) {
+      m = max(m, x[k]);
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, x[k], o);
+        if (lane >= o) x[k] += y;
+      }
+      x[k] += run;
+      run = __shfl_sync(0xffffffffu, x[k], 31);
     }
-    *maxlen = mm;
+    if (lane == 0) warp_sum[buf][w] = run;
+    __syncthreads();   // two buffers: the next tile's sums never meet a reader of this tile's
+    int s = warp_sum[buf][lane];   // kScanThreads / 32 == 32 warps, one per lane
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, s, o);
+      if (lane >= o) s += y;
+    }
+    const int before = __shfl_sync(0xffffffffu, s, (w + 31) & 31), total = __shfl_sync(0xffffffffu, s, 31);
+    const int add = carry + (w ? before : 0);
+#pragma unroll
+    for (int k = 0; k < kScanPer; k++)
+      if (at + 32 * k < len) rp[at + 32 * k] = x[k] + add;
+    carry += total;
   }
+  m = __reduce_max_sync(0xffffffffu, m);
+  if (lane == 0) warp_max[w] = m;
   __syncthreads();
-  long long run = part[t];
-  for (int64_t i = b; i < e; i++) {
-    run += rp[i];
-    rp[i] = (int)run;
+  if (w == 0) {
+    m = __reduce_max_sync(0xffffffffu, warp_max[lane]);
+    if (lane == 0) *maxlen = m;
   }
 }
+static_assert(kScanThreads == 1024, "k_tr_scan: one warp sum per lane");
 
 // every entry into its column's segment at a free place (any order), keyed by its index q
 __global__ void k_tr_fill(const int* __restrict__ ci, const double* __restrict__ v, int64_t nnz,
@@ -297,7 +317,7 @@ cudaError_t transpose_layout(const Csr& M, int* rpT, int* maxlen, cudaStream_t s
   if (e != cudaSuccess) return e;
   const int blocks = (int)std::min<int64_t>((M.nnz + kThreads - 1) / kThreads + 1, 152 * 8);
   if (M.nnz > 0) k_tr_count<<<blocks, kThreads, 0, s>>>(M.ci, M.nnz, rpT);
-  k_tr_scan<<<1, kThreads, 0, s>>>(rpT, M.cols + 1, maxlen);
+  k_tr_scan<<<1, kScanThreads, 0, s>>>(rpT, M.cols + 1, maxlen);
   return cudaGetLastError();
 }
 
@@ -310,6 +330,76 @@ cudaError_t transpose_fill(const Csr& M, const int* rpT, int* cur, int* ciT, dou
   k_tr_fill<<<qb, kThreads, 0, s>>>(M.ci, M.v, M.nnz, rpT, cur, ciT, vT);
   k_tr_sort<<<cb, kThreads, 0, s>>>(rpT, M.cols, ciT, vT);
   k_tr_rows<<<qb, kThreads, 0, s>>>(M.rp, M.rows, M.nnz, ciT);
+  return cudaGetLastError();
+}
+
+// ---- explicit entries of sum_f B_f^T B_f (thin factor terms).  Row j lists, for each term, each entry (r, j) of B_f
+// in the order of B_f^T's row and each entry of B_f's row r.  Entry e of B_f^T starts len(r) entries, so the
+// scan S_f of these lengths gives the row pointers (sum_f S_f at the row pointers of B_f^T) and every
+// entry's place; no scan over the n rows is needed.  Bound by launch latency: 0.08 ms for S of the n = 1e6 CQP
+// (9e4 entries), 5 ms on the host with the upload of its row pointers.
+// off[e + 1] = length of the row of B that entry e of B^T names (off[0] = 0)
+__global__ void k_thin_len(const int* __restrict__ rpB, const int* __restrict__ ciT, int64_t nnz, int* __restrict__ off) {
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nnz; e += stride) {
+    const int r = ciT[e];
+    off[e + 1] = rpB[r + 1] - rpB[r];
+  }
+}
+
+__global__ void k_thin_rp(const ThinTerms T, int64_t n, int* __restrict__ rp) {
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j <= n; j += stride) {
+    int at = 0;
+    for (int f = 0; f < T.count; f++) at += T.off[f][T.BT[f].rp[j]];
+    rp[j] = at;
+  }
+}
+
+// the entries that entry e of B_f^T starts, one thread each (a row of a thin factor is short)
+__global__ void k_thin_fill(const ThinTerms T, int f, int64_t n, const int* __restrict__ rp, int* __restrict__ ci,
+                            double* __restrict__ v) {
+  const Csr &B = T.B[f], &BT = T.BT[f];
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < BT.nnz; e += stride) {
+    int64_t lo = 0, hi = n - 1;   // e's row of B_f^T: the last j with rp[j] <= e
+    while (lo < hi) {
+      const int64_t mid = (lo + hi + 1) / 2;
+      if (BT.rp[mid] <= e) lo = mid;
+      else hi = mid - 1;
+    }
+    int64_t q = (int64_t)rp[lo] + T.off[f][e] - T.off[f][BT.rp[lo]];
+    for (int g = 0; g < f; g++) q += T.off[g][T.BT[g].rp[lo + 1]] - T.off[g][T.BT[g].rp[lo]];
+    const int r = BT.ci[e];
+    const double x = BT.v[e];
+    for (int i = B.rp[r]; i < B.rp[r + 1]; i++, q++) {
+      ci[q] = B.ci[i];
+      v[q] = x * B.v[i];
+    }
+  }
+}
+
+cudaError_t thin_layout(const ThinTerms& T, int64_t n, int* rp, int* maxlen, cudaStream_t s) {
+  for (int f = 0; f < T.count; f++) {
+    const int64_t nnz = T.BT[f].nnz;
+    const int blocks = (int)std::min<int64_t>((nnz + kThreads - 1) / kThreads + 1, 152 * 8);
+    const cudaError_t e = cudaMemsetAsync(T.off[f], 0, sizeof(int), s);
+    if (e != cudaSuccess) return e;
+    if (nnz == 0) continue;
+    k_thin_len<<<blocks, kThreads, 0, s>>>(T.B[f].rp, T.BT[f].ci, nnz, T.off[f]);
+    k_tr_scan<<<1, kScanThreads, 0, s>>>(T.off[f], nnz + 1, maxlen);
+  }
+  k_thin_rp<<<(int)std::min<int64_t>(n / kThreads + 1, 152 * 8), kThreads, 0, s>>>(T, n, rp);
+  return cudaGetLastError();
+}
+
+cudaError_t thin_fill(const ThinTerms& T, int64_t n, const int* rp, int* ci, double* v, cudaStream_t s) {
+  for (int f = 0; f < T.count; f++) {
+    const int64_t nnz = T.BT[f].nnz;
+    if (nnz == 0) continue;
+    const int blocks = (int)std::min<int64_t>((nnz + kThreads - 1) / kThreads, 152 * 8);
+    k_thin_fill<<<blocks, kThreads, 0, s>>>(T, f, n, rp, ci, v);
+  }
   return cudaGetLastError();
 }
 

@@ -27,4 +27,15 @@ cudaError_t tile_fill(const Csr& M, int W, int ntile, const int* slot, const int
 cudaError_t transpose_layout(const Csr& M, int* rpT, int* maxlen, cudaStream_t s);
 cudaError_t transpose_fill(const Csr& M, const int* rpT, int* cur, int* ciT, double* vT, cudaStream_t s);
 
+// CSR matrix sum_f B_f^T B_f (duplicates kept) of factor terms on the device with their transposes:
+// thin_layout fills off[f] (BT[f].nnz + 1 each) and rp (n + 1), using maxlen as scratch; thin_fill then writes
+// ci / v (sum over all rows of B_f of their squared lengths, < 2^31, entries).
+struct ThinTerms {
+  int count = 0;
+  Csr B[kMaxFac], BT[kMaxFac];
+  int* off[kMaxFac] = {nullptr};
+};
+cudaError_t thin_layout(const ThinTerms& T, int64_t n, int* rp, int* maxlen, cudaStream_t s);
+cudaError_t thin_fill(const ThinTerms& T, int64_t n, const int* rp, int* ci, double* v, cudaStream_t s);
+
 }  // namespace hprqp
