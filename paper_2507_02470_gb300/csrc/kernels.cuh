@@ -850,8 +850,11 @@ __device__ __forceinline__ void rows_body(const Args& a, const Handles& hd) {
   constexpr bool RED = (VAR != VAR_PLAIN) && !FUSED;   // the variant carries reduction code
   const int64_t rows = (KIND == K_A1 || KIND == K_APPLY_A || KIND == K_POWER_A) ? a.m : a.n;
   constexpr bool OVER_M = KIND == K_A1 || KIND == K_APPLY_A || KIND == K_POWER_A;
-  const int R = OVER_M ? a.rowsA : kChunk;
-  const int64_t nchunks = (rows + R - 1) / R;
+  // rows per block pass: fixed at compile time for the SELL form, whose slices are laid out by kChunk (the tuner
+  // takes it for no other rowsA); the count of passes by a 32-bit division (rows < 2^31)
+  constexpr bool FEW = OVER_M && G != -1;
+  const int R = FEW ? a.rowsA : kChunk;
+  const int64_t nchunks = FEW ? (int64_t)((unsigned)(rows + R - 1) / (unsigned)R) : (rows + kChunk - 1) / kChunk;
   const double sigma = C->sigma, s = C->s, slA = C->slA, inv_slA = C->inv_slA;
   const int mode = C->mode;
   // the fused passes apply the Halpern step that follows this one (the weights the controller
@@ -899,7 +902,7 @@ __device__ __forceinline__ void rows_body(const Args& a, const Handles& hd) {
     if constexpr (G != 1) __syncthreads();
     // ---- phase 2: thread per row, full warps
     const int64_t j = row0 + threadIdx.x;
-    if (j < rows && (!OVER_M || (int)threadIdx.x < R)) {
+    if (j < rows && (!FEW || (int)threadIdx.x < R)) {
       const double r0 = rs0[threadIdx.x];
       if (KIND == K_Q1) {
         const double* src = HA ? V.wh : V.wb;
