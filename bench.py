@@ -71,7 +71,7 @@ def workload(name: str):
     if name == "qap":
         return qpgen.qap_relaxation(d=256, seed=0), \
             ("QAP relaxation (Sec. 4.5) d=256: n=65536, m=512, Q = Bhat(x)Ahat - I(x)S - T(x)I matrix-free "
-             "(two FP64 contractions per product)")
+             "(FP64-accurate digit products on the tensor cores)")
     raise SystemExit(f"unknown workload {name}")
 
 
@@ -453,7 +453,8 @@ def algorithmic(qp, tiled=False):
     for t in qp.qterms:
         if t.kind == "qap":
             # Ahat X (d^3 FMAs), then [T1 | S | X] [Bhat; -X; -T] (3 d^3): the four d x d
-            # matrices, x twice, T1 written and read, the result written
+            # matrices, x twice, T1 written and read, the result written (formed from digit
+            # products on the tensor cores from d = QAP_TC_MIN_D on: see roofline)
             d = int(round(np.sqrt(n)))
             qap_bytes += 8 * 9 * d * d
             qap_flops += 4 * d ** 3
@@ -531,7 +532,12 @@ def fp64_peak(pk):
                                    f"(probe at {r['sm_mhz']:.0f} MHz)")
 
 
-def roofline(prof, qp, pk, pk_src, traffic, tiled=False, iter_s=None, fp64=None):
+# csrc/qap_tc.cu: the smallest d of the tensor-core form, and the digit products kept per operand pair
+QAP_TC_MIN_D = 8
+QAP_DIGIT_PRODUCTS = 34
+
+
+def roofline(prof, qp, pk, pk_src, traffic, tiled=False, iter_s=None, fp64=None, launches_per_iter=None):
     """Roofline of the dominant kernel (the longest mean CUDA-event duration over plain steps)
     by its algorithmic bytes and FP64 operations per launch, against the measured HBM copy rate
     and the FP64 issue peak; plus the whole iteration by iteration_bytes() over the measured
@@ -560,6 +566,17 @@ def roofline(prof, qp, pk, pk_src, traffic, tiled=False, iter_s=None, fp64=None)
     r.update({"traffic": tr, "kernel": name, "ms_per_launch": round(ms, 5), "alg_bytes": int(b), "alg_fp64": int(f),
               "peak_source": f"hbm {pk_src} (MEASURED_PEAKS.json, of measured); fp64 {fp64_src}",
               "all_kernels_ms": {k: round(v, 5) for k, v in prof.items() if v > 0}})
+    d = max((int(round(np.sqrt(qp.n))) for t in qp.qterms if t.kind == "qap"), default=0)
+    if d >= QAP_TC_MIN_D and name in ("pre1", "pre2", "prew"):
+        # the product runs as QAP_DIGIT_PRODUCTS signed 8-bit digit products on the BF16 tensor cores
+        tf = QAP_DIGIT_PRODUCTS * 2 * 4 * d ** 3 / (ms * 1e-3) / 1e12
+        peak = float(pk.get("bf16_tflops", 1900.0))
+        r.pop("alu_frac", None)
+        r.update({"bound": "latency", "achieved": round(tf, 2), "peak": peak, "unit": "TFLOP/s (BF16 digit products)",
+                  "frac": round(tf / peak, 4), "hbm_frac": round(frac_h, 4), "fp64_equiv_gops": round(ops, 2)})
+    if launches_per_iter is not None and launches_per_iter < 1:
+        r["note"] = ("the timed solves run in the resident kernel; all_kernels_ms are the separate kernels that "
+                     "hprqp_profile launches")
     if iter_s:
         ib = iteration_bytes(qp)
         r["iteration"] = {"alg_bytes": int(ib), "us": round(iter_s * 1e6, 2),
@@ -792,7 +809,8 @@ def main():
     nfac = sum(1 for t in qp.qterms if t.kind == "factor")
     iter_s = statistics.median((k["solve_seconds"] - k["power_seconds"]) / k["iters"] for k in kkts)
     roof = roofline(prof, qp, pk, pk_src, traffic_table(args.workload), tiled=nfac > 0 and kk["tiled_terms"] == nfac,
-                    iter_s=iter_s, fp64=fp64_peak(pk))
+                    iter_s=iter_s, fp64=fp64_peak(pk),
+                    launches_per_iter=launches / max(1, sum(iters_per_step)))
 
     # end to end through the C ABI with host buffers: create (H2D), solve, get (D2H)
     host = {k: (torch.from_numpy(np.ascontiguousarray(v)).pin_memory() if isinstance(v, np.ndarray) else v)

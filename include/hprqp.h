@@ -57,9 +57,11 @@ typedef enum hprqp_qkind {
   HPRQP_Q_QAP = 6            /* Q vec(X) += vec(Ahat X Bhat - S X - X T) for d x d X with
                                 n = d^2, vec(X)[i + j d] = X[i][j] (the QAP relaxation of
                                 Sec. 4.5): p = d, dense = Ahat, Bhat, S, T (symmetric d x d,
-                                4 d^2 values one after another); applied as two FP64
-                                contractions, Ahat X then [Ahat X | S | X][Bhat; -X; -T];
-                                at most one such term; not with launch_mode 3 */
+                                4 d^2 values one after another); applied as Ahat X,
+                                then [Ahat X | S | X][Bhat; -X; -T]: on the tensor cores
+                                at FP64 accuracy (autotune 1 and d >= 8; a row or column of
+                                an operand with a non-finite entry gives NaN), else as FP64
+                                contractions; at most one such term; not with launch_mode 3 */
 } hprqp_qkind;
 
 typedef enum hprqp_phi {
@@ -127,7 +129,11 @@ typedef struct hprqp_params {
   hprqp_alloc_fn alloc;      /* optional allocator hooks (see above) */
   hprqp_free_fn free;
   void* alloc_ctx;
-  int32_t launch_mode;       /* 0 (default): CUDA graphs with conditional nodes: whole check
+  int32_t launch_mode;       /* 0 (default): a problem whose state fits the SMs' shared memory
+                                (n up to about 190,000; Q present, no QAP or tiled term,
+                                schedule options at their defaults) is solved by one
+                                resident launch per 2^15 steps; any other by
+                                CUDA graphs with conditional nodes: whole check
                                 periods through a graph whose step variants are fixed by
                                 position (see fixed_schedule), the rest through a graph whose
                                 conditional nodes pick each step's variant on the device;

@@ -1249,9 +1249,8 @@ static hprqp_status create_impl(hprqp_handle* h, int64_t n, int64_t m, const hpr
     for (int f = 0; f < QD.nfac; f++)
       if (!big || QD.fact[f].nnz > big->nnz) big = &QD.fact[f];
     P.gQ = big ? tune_G(h, *big, kChunk, P.gridN, ain, aout, 1) : 1;
-    // Q's CSR-like parts are only thin factors formed on demand: one lane per row (their few
-    // entries gain nothing from more lanes, and the bare-SpMV probe cannot see the on-demand
-    // products).  A SELL copy of B^T, which packs a chunk's entries into one warp, measured
+    // Q's CSR-like parts are only thin factors (their explicit entries): one lane per row (their few
+    // entries gain nothing from more lanes).  A SELL copy of B^T, which packs a chunk's entries into one warp, measured
     // slower on the n = 1e6 CQP (longer chain of dependent loads per entry).
     {
       bool only_inl = QD.nfac > 0 && !QD.csr.rows;

@@ -77,7 +77,7 @@ struct QDev {
   const double* dense[kMaxDense] = {nullptr};   // F_g row-major p x n
   int64_t toff[kMaxFac + kMaxDense] = {0};
   // QAP term (Sec. 4.5): Ahat, Bhat, S, T (d x d each, contiguous); its product Q_qap x is
-  // formed before a pass (the FP64 contractions of qap.cu) into the intermediate buffer at
+  // formed before a pass (qap_tc.cu, or the FP64 contractions of qap.cu) into the intermediate buffer at
   // qap_off, like B_f x
   int64_t qap_d = 0;
   const double* qap = nullptr;
