@@ -8,7 +8,10 @@
 // of the matrices lies in shared memory; only the vectors that the products gather from
 // (wbar_{1/2}, v, ybar, w, and the factor products t) go through L2, each followed by a grid
 // barrier.  A plain step is E (elementwise) | Q wbar_{1/2}, v | A v, ybar | A^T ybar, w | Q w, E of the
-// next step: four barriers, two more when Q has a factor product to form first.  The arithmetic per
+// next step: four barriers, two more when Q has a factor product to form first.  Without rows of A a
+// step is E | Q wbar_{1/2} with the one barrier between them, and wbar_{1/2} lies in two vectors in turn: a
+// block that is done with its products stores the next step's while others still gather this one's, and
+// the barrier keeps it from getting further ahead.  The arithmetic per
 // row is that of the fused passes of kernels.cuh; a step that evaluates R~ or the stopping rule takes
 // the unfused form, like there.  Every block sums the blocks' partial results itself, in block order,
 // and runs the controller on its own copy: no broadcast, and the same decisions everywhere.
@@ -609,9 +612,10 @@ __device__ __forceinline__ void init_ctx(Ctx<CL>& c) {
   c.mr = min((int)c.a.m - c.i0, c.p.rm);
 }
 
-// E: the pending Halpern or restart update of (x, w_Q, Q w, A^* y) and eqs. (3.1)-(3.3) on the own rows
+// E: the pending Halpern or restart update of (x, w_Q, Q w, A^* y) and eqs. (3.1)-(3.3) on the own rows,
+// wbar_{1/2} into the gathered vector `half`
 template <bool CL>
-__device__ void elementwise(const Ctx<CL>& c, const Step& st) {
+__device__ void elementwise(const Ctx<CL>& c, const Step& st, double* half) {
   const int mode = st.mode, ttest = st.ttest;
   const double ha = st.ha, hb = st.hb;
   const Args& a = c.a;
@@ -645,7 +649,7 @@ __device__ void elementwise(const Ctx<CL>& c, const Step& st) {
     c.n_row(SXH)[i] = xh;
     c.n_row(SWH)[i] = wh;
     if (!HA) c.n_row(SWB)[i] = wh;
-    c.put(c.wh + j, wh);
+    c.put(half + j, wh);
     if (ttest) {
       c.put(c.xb + j, xbar);
       V.zb[j] = (xbar - rz) * st.isigma;
@@ -789,7 +793,10 @@ __global__ void __launch_bounds__(MT, 1)
   if (CL) all_sync(c);   // a block's shared memory may be written once it runs
   if (c.tid == 0) S.st[1] = step_of(S.C);
   __syncthreads();
-  elementwise(c, S.st[1]);
+  // wbar_{1/2} of step `it` as the products gather it: with m = 0 no barrier lies between them and E of the next
+  // step, which stores into the other vector (v, unused then)
+  auto half = [&](long long it) { return HA || (it & 1) ? c.wh : c.v; };
+  elementwise(c, S.st[1], half(1));
   bool ok = true;
   for (long long it = 1;; it++) {
     // E of this step is done
@@ -799,17 +806,18 @@ __global__ void __launch_bounds__(MT, 1)
     const bool plain = !rtest && !ttest;
     const bool fused = plain && HA && it < r.steps;
     const double* x1 = ttest ? c.xb : nullptr;
+    const double* wh = half(it);
     // a plain step takes no decision: the controller moves on to the next step meanwhile
     if (!(ok = all_sync(c, [&] { if (plain) advance_plain(S.C, st, next, c.tid & 31); }))) break;
     if (pre) {
-      factor_rows(c, c.wh, x1, c.t1, c.t1 + Q.tlen, true);
+      factor_rows(c, wh, x1, c.t1, c.t1 + Q.tlen, true);
       if (!(ok = all_sync(c))) break;
     }
     // Q wbar_{1/2} (and Q xbar), v
-    q_sums(c, c.wh, x1, c.t1, c.t1 + Q.tlen, true);
+    q_sums(c, wh, x1, c.t1, c.t1 + Q.tlen, true);
     for (int i = c.tid; i < c.nr; i += c.T) {
       const int j = c.j0 + i;
-      const double qwh = c.rs0()[i] + q_bands(c, j, c.wh);
+      const double qwh = c.rs0()[i] + q_bands(c, j, wh);
       if (HA) c.put(c.v + j, fma(st.sigma, c.n_row(SQW)[i] - qwh, c.n_row(SXH)[i]));
       else c.n_row(SQWB)[i] = qwh;
       if (rtest) V.Qwh[j] = qwh;
@@ -939,7 +947,7 @@ __global__ void __launch_bounds__(MT, 1)
       if (c.tid == 0) next = step_of(S.C);
       __syncthreads();
     }
-    if (!fused) elementwise(c, next);
+    if (!fused) elementwise(c, next, half(it + 1));
   }
   // no block still gathers from the vectors that are stored below (or from a copy in a block that ends)
   if (!ok || !all_sync(c)) return;
