@@ -311,7 +311,7 @@ class Solver:
         self._keep = []
 
     def set_wait_polls(self, polls):
-        """launch_mode 3: polls of one grid-barrier wait before the solve gives up (0: default)."""
+        """Polls of one grid-barrier wait before a solve (launch_mode 3, resident launches) gives up (0: default)."""
         self._check(lib().hprqp_set_wait_polls(self.h, int(polls)))
 
     def set_lambda(self, lambda_A, lambda_Q):

@@ -1552,6 +1552,7 @@ static double power_start_scale(hprqp_handle* h, int which) {
 static ResRun resident_run(const hprqp_handle* h, long long steps) {
   ResRun r;
   r.steps = steps;
+  if (h->prm.wait_polls > 0) r.spin = (unsigned)h->prm.wait_polls;
   r.flags = h->res_flags;
   r.err = reinterpret_cast<int*>(h->res_flags + 1);
   r.part = h->res_part;

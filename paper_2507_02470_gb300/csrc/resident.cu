@@ -24,7 +24,7 @@
 //   * larger problems use up to one block per SM and vectors in L2.  The barrier is a counter: one
 //     release-add per block, one thread per block polls with acquire loads.  On 152 blocks that is 2640
 //     cycles; flags read by every block took 8000, and a fence per polling thread more.  Every wait
-//     is bounded; a block whose wait gives up sets the error flag and leaves, the others follow at their
+//     is bounded (ResRun::spin polls); a block whose wait gives up sets the error flag and leaves, the others follow at their
 //     next barrier, and the host reports HPRQP_TIMEOUT.
 // FP64 (measured): a dependent FMA takes 64 cycles, as long as its issue slot, so four warps fill an
 // SM's FP64 pipe; a division takes 640.
@@ -38,7 +38,6 @@
 namespace hprqp {
 namespace {
 
-constexpr unsigned kSpin = 1u << 22;   // polls of one wait (a few seconds; each is a round trip to L2)
 constexpr int kTerm = 16;              // sums of one reduction: 12 end-of-step, 4 of the y-step
 
 // rows of the shared-memory state, rn values each
@@ -142,7 +141,7 @@ __device__ __forceinline__ bool all_sync(Ctx<CL>& x, F work) {
     for (unsigned i = 0;; ++i) {
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(x.r.flags) : "memory");
       if ((int)(v - x.epoch) >= 0) break;
-      if (i >= kSpin || ((i & 1023u) == 1023u && *(volatile int*)x.r.err)) {
+      if (i >= x.r.spin || ((i & 1023u) == 1023u && *(volatile int*)x.r.err)) {
         atomicExch(x.r.err, 1);
         bad = 1;
         break;

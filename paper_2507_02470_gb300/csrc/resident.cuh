@@ -30,10 +30,13 @@ struct ResPlan {
   size_t smem = 0;           // dynamic shared memory of a block
 };
 
+constexpr unsigned kResSpin = 1u << 22;   // polls of one wait, unless asked otherwise (a few seconds; each is a round trip to L2)
+
 // Per launch: at most `steps` inner steps; flags: the barrier's counter, followed by the error word; part:
-// 2 x B x 16 partial sums; lam: 2 results of the power methods.
+// 2 x B x 16 partial sums; lam: 2 results of the power methods; spin: polls of one wait of the grid barrier.
 struct ResRun {
   long long steps = 0;
+  unsigned spin = kResSpin;
   unsigned* flags = nullptr;
   int* err = nullptr;
   double* part = nullptr;
