@@ -1285,7 +1285,7 @@ static cudaError_t launch_bucket(hprqp_batch* b, int bk, int beg, int cnt, int t
   const Sched& S = b->sched;
   const KFn k = batch_kernel(fs, small_p(S, bk));
   const size_t smem = launch_smem(S, bk, fs, cnt, threads, sms);
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = shared_memory_limit((const void*)k);   // the same for every bucket and batch: other threads launch k too
   int occ = 0;
   if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, threads, smem);
   if (e != cudaSuccess) return e;
@@ -1343,7 +1343,7 @@ static hprqp_status batch_autotune(hprqp_batch* b, int sms) {
         const KFn k = batch_kernel(fs != 0, small_p(S, bk));
         const size_t smem = bucket_smem(S, bk, fs != 0);
         int occ = 0;
-        BCU(b, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        BCU(b, shared_memory_limit((const void*)k));
         BCU(b, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, G, smem));
         if (occ < 1) continue;   // no block of this shape fits an SM
         const int sample = std::min(cnt, sms * occ);

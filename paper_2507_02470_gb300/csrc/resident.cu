@@ -1078,9 +1078,11 @@ PowerKernel power_kernel(const ResPlan& p) {
                    : p.T > 512 ? k_resident_power<false, kResThreads> : k_resident_power<false, 512>;
 }
 
+// Lets kernel k take any plan's shared memory and cluster.  The limits belong to the kernel, not to a launch: they are
+// set to the same values every time, so that handles with other plans may launch k from other threads meanwhile.
 cudaError_t setup(const ResPlan& p, const void* k) {
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
-  if (e == cudaSuccess && p.cluster && p.B > 8) e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  cudaError_t e = shared_memory_limit(k);
+  if (e == cudaSuccess && p.cluster) e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   return e;
 }
 

@@ -620,6 +620,15 @@ __global__ void __launch_bounds__(kThreads) k_spmv_probe(Csr M, int R, const dou
 }
 
 // the factor pre-pass t = B_f ain (which = 3) at G lanes per row, for the schedule autotuner
+cudaError_t shared_memory_limit(const void* k) {
+  int dev = 0, most = 0;
+  cudaFuncAttributes f;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&f, k);
+  return e != cudaSuccess ? e : cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)f.sharedSizeBytes);
+}
+
 cudaError_t launch_pre_probe(const Args& a, int G, int grid, cudaStream_t s) {
   prek(G, 0)<<<grid, kThreads, 0, s>>>(a, 3);
   return cudaGetLastError();

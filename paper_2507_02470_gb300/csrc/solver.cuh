@@ -130,6 +130,8 @@ cudaError_t launch_power_iter(const Args& a, const Plan& p, int which, int i, cu
 int kernels_per_power_iter(const Args& a, int which);
 cudaError_t launch_power_init(const Args& a, const Plan& p, int which, cudaStream_t s);
 cudaError_t launch_zbar(const Args& a, const Plan& p, cudaStream_t s);
+// Raises kernel k's limit of dynamic shared memory to what the current device leaves beside k's static part
+cudaError_t shared_memory_limit(const void* k);
 cudaError_t launch_spmv_probe(const Csr& M, int G, int R, int grid, const double* x, double* y, cudaStream_t s);
 cudaError_t launch_pre_probe(const Args& a, int G, int grid, cudaStream_t s);
 // shared-memory-tiled factor products (tiled.cu): t = B_f x, then (which != 2) u = B_f^T t,
