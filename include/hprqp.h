@@ -59,9 +59,10 @@ typedef enum hprqp_qkind {
                                 Sec. 4.5): p = d, dense = Ahat, Bhat, S, T (symmetric d x d,
                                 4 d^2 values one after another); applied as Ahat X,
                                 then [Ahat X | S | X][Bhat; -X; -T]: on the tensor cores
-                                at FP64 accuracy (autotune 1 and d >= 8; a row or column of
-                                an operand with a non-finite entry gives NaN), else as FP64
-                                contractions; at most one such term; not with launch_mode 3 */
+                                (autotune 1 and d >= 8; every element within the error bound
+                                of the FP64 sums, d 2^-53 |Ahat| |X| for the first product and
+                                3 d 2^-53 of the magnitudes added for the second), else as
+                                FP64 contractions; at most one such term; not with launch_mode 3 */
 } hprqp_qkind;
 
 typedef enum hprqp_phi {

@@ -12,20 +12,32 @@
 //     q = sum_i d_i 256^(6-i), d_i in [-128, 128]: a BF16 value holds a digit exactly;
 //   * P_s = sum over i + j = s and over 64 values of k of d_i(A) d_j(B) is at most 7 * 64 * 2^14 < 2^23, so the
 //     FP32 accumulators (one 64-column block of tensor memory per s) are exact; s = 0 .. 7 are kept (34 digit
-//     products), the rest lies below 2^-57 of the row's and column's maxima;
+//     products);
 //   * the P_s are joined in two 64-bit integers (s < 4 and s >= 4), chunks of k added there, so the result does
 //     not depend on any order; the last step is one FP64 rounding of the exact sum.
-// The products are closer to the exact ones than the FP64 contraction's (relative to a long double product,
-// 2-norm: 8e-17 against 6e-16 at d = 96; d = 256 on the GPU: see tests/test_gpu_qap_tc.py).
+// Accuracy, element by element.  Let a be the power of two at or below the largest magnitude of a left operand's row
+// and b that of a right operand's column.  An entry is off by at most 2^-55 a (half a unit of q), so a term of
+// a product by less than 1.02 2^-53 a b, the dropped digit products (5 * 2^46 units of 2^-108 a b) among it, and
+// an element of k terms by less than 1.02 k 2^-53 a b.  An FP64 sum of the terms may be off by k 2^-53
+// (|A| |B|)_ij.  So where |(A B)_ij| >= 1.02 a b the digits are no worse, whatever the data; where it is smaller (a
+// row's or column's few large entries meet small ones, or the sum cancels) the element is formed anew, in
+// FP64, by the kernel that joins it (dot8).  T1 is held to this element by element; the three products of the result
+// together, as their one FP64 sum would be.  Rows and columns that are not finite take the same way, so that NaN
+// and infinities come out as FP64 gives them.  Share of elements formed anew on the iterates of the
+// relaxation (d = 16 to 128, 1 to 400 steps): none of Q w and Q w_{1/2}, 0.1 to 0.5 of Q xbar (tests only).
+// In the 2-norm the digits are closer than the FP64 contraction (relative to a long double product: 8e-17
+// against 6e-16 at d = 96).
 //
 // One product is five kernels: k_slice_x (digits of X by rows and by columns), k_fix on Ahat X, S X and X T at
 // once, k_slice_t1 (joins Ahat X, digits by rows), k_fix on T1 Bhat, k_join.  A CTA of k_fix owns a 128 x 64
 // tile of one product and one or several chunks of 64 k's; a chunk's digits of both operands (172 KB) are
 // fetched with 14 TMA loads behind one mbarrier and multiplied by 136 tcgen05.mma.
 // us per product before a pass, FP64 contractions (qap.cu) / this path: d = 9: 49 / 43, 32: 85 / 43, 64: 162 / 49,
-// 128: 186 / 53, 256: 189 / 57, 400: 728 / 175; at d = 256 the two k_fix take 13 us each.  Below d = 8 one
-// FP64 tile is as fast.
+// 128: 186 / 53, 256: 189 / 58, 400: 728 / 175; at d = 256 the two k_fix take 13 us each.  Below d = 8 one
+// FP64 tile is as fast.  With every element formed anew (rows and columns over 20 orders of magnitude) a product takes
+// 21 us more at d = 64, 40 at 128, 98 at 256: no longer than the contractions.
 #include <algorithm>
+#include <cfloat>
 #include <vector>
 
 #include "qap_tc.cuh"
@@ -44,20 +56,24 @@ constexpr uint32_t kABytes = kBM * kBK * 2, kBBytes = kBN * kBK * 2;
 constexpr uint32_t kFixSmem = 1024 + kDig * (kABytes + kBBytes);
 
 // ------------------------------------------------------------------------------------ digits
-// biased exponent of v (2047: not finite), by its upper half alone
-__device__ __forceinline__ int exponent(double v) { return (int)(((unsigned)__double2hiint(v) >> 20) & 0x7ffu); }
+// biased exponent of v (2047: not finite; 1 for subnormals, which share its unit; 0: v is 0)
+__device__ __forceinline__ int exponent(double v) {
+  const unsigned mag = (unsigned)__double2hiint(v) & 0x7fffffffu;
+  return mag >> 20 ? (int)(mag >> 20) : (mag | (unsigned)__double2loint(v)) != 0u;
+}
 
-// 2^(e - 1057): a row's scale; NaN for a row that is not finite, so that its products are NaN
+// 2^(e - 1057): a row's scale; 0 for a row of zeros; NaN for a row that is not finite, so that its products are NaN
 __device__ __forceinline__ double row_scale(int e) {
+  if (e == 0) return 0.0;
   return e == 2047 ? __longlong_as_double(0x7ff8000000000000ll) : scalbn(1.0, e - 1057);
 }
 
-// round(v 2^(1077 - e)) for a finite v of exponent <= e (FP64 subnormals count as 0)
+// round(v 2^(1077 - e)) for a finite v of exponent <= e
 __device__ __forceinline__ long long fixed(double v, int e) {
   const int ev = exponent(v);
   if (ev == 0 || ev == 2047 || e == 2047) return 0;
-  const unsigned hi = (unsigned)__double2hiint(v);
-  const long long man = ((long long)((hi & 0xfffffu) | 0x100000u) << 32) | (unsigned)__double2loint(v);
+  const unsigned hi = (unsigned)__double2hiint(v), top = (hi & 0x7ff00000u) ? 0x100000u : 0u;
+  const long long man = ((long long)((hi & 0xfffffu) | top) << 32) | (unsigned)__double2loint(v);
   const int sh = e - ev - 2;   // man 2^(2 - (e - ev))
   long long q;
   if (sh <= 0) q = man << -sh;
@@ -149,8 +165,11 @@ __global__ void __launch_bounds__(kFarThreads) k_slice_x(const double* x, QapTcD
 }
 
 // ------------------------------------------------------------------------------------ products
-// element (i, j) of product `prod`, from its partial sums
-__device__ __forceinline__ double join(const QapTcDev& q, int prod, int a, int b, int i, int j) {
+// biased exponent of |v| by its upper half (0 for subnormals too)
+__device__ __forceinline__ int field(double v) { return (int)(((unsigned)__double2hiint(v) >> 20) & 0x7ffu); }
+
+// element (i, j) of product `prod`, from its partial sums; size: field() of its row's and its column's scale, summed
+__device__ __forceinline__ double join(const QapTcDev& q, int prod, int a, int b, int i, int j, int& size) {
   const size_t dd = (size_t)q.d * q.d;
   const long long* p = q.part + (size_t)prod * q.groups * 2 * dd + (size_t)j * q.d + i;
   long long h[kGroups], l[kGroups];   // all loads in flight
@@ -160,29 +179,113 @@ __device__ __forceinline__ double join(const QapTcDev& q, int prod, int a, int b
     l[g] = g < q.groups ? __ldcg(p + (2 * g + 1) * dd) : 0;
   }
   const long long hi = (h[0] + h[1]) + (h[2] + h[3]), lo = (l[0] + l[1]) + (l[2] + l[3]);
-  // hi < 2^53 and lo < 2^53 are exact in FP64
-  // the smaller scale first: a product in FP64's range does not overflow on the way to it
+  // |hi| < 2^45 per chunk of k: exact in FP64 up to 2^8 chunks (d = 16,384), rounded once beyond, like the result.
+  // |lo| < 2^47 per chunk: from 2^6 chunks on it may round too, by less than 2^-53 of it, where an element that
+  // is kept is 2^68 at least.
+  // The smaller scale first: a product in FP64's range does not overflow on the way to it.
   const double v = fma((double)hi, 4294967296.0, (double)lo), sa = q.scale[a][i], sb = q.scale[b][j];
+  size = field(sa) + field(sb);
   return sa < sb ? v * sa * sb : v * sb * sa;
+}
+// Whether a finite sum of up to three products, the largest of exponent field `top`, reaches the sum of their 1.02 a b,
+// by exponents alone (FP64 operations on every element took 5 us of a product at d = 256): a b is at most
+// 2^(size + 68 - 2046), three times 1.02 of it less than four.
+__device__ __forceinline__ bool reaches(int top, int size) { return top < 2047 && top >= size + 68 + 2 - 1023; }
+// 1.02 a b (a is 2^34 of the row's scale); 0 for a row or column of zeros
+__device__ __forceinline__ double least(const QapTcDev& q, int a, int b, int i, int j) {
+  return 1.02 * (17179869184.0 * q.scale[a][i]) * (17179869184.0 * q.scale[b][j]);
+}
+
+// For each lane with bad set: term(k, src) summed over k < d in FP64, src the lane whose element it is; returned in
+// that lane (others: `keep`).  Eight lanes an element, four elements of the warp at a time, two running sums a lane
+// of eight loads in flight: a fixed order.  All lanes call it.
+template <class F>
+__device__ __forceinline__ double dot8(bool bad, double keep, int d, F term) {
+  const unsigned all = 0xffffffffu, mask = __ballot_sync(all, bad);
+  const int lane = threadIdx.x & 31, l = lane & 7, grp = lane >> 3, rank = __popc(mask & ((1u << lane) - 1u));
+  unsigned left = mask;
+  for (int round = 0; left; round++) {
+    int src = -1;   // the element of this group of lanes
+#pragma unroll
+    for (int g = 0; g < 4; g++) {
+      if (g == grp && left) src = __ffs(left) - 1;
+      left &= left - 1u;
+    }
+    double s0 = 0.0, s1 = 0.0;
+    if (src >= 0) {
+      int k = l;
+#pragma unroll 4
+      for (; k + 8 < d; k += 16) {
+        s0 = term(s0, k, src);
+        s1 = term(s1, k + 8, src);
+      }
+      if (k < d) s0 = term(s0, k, src);
+    }
+    double s = s0 + s1;
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(all, s, o);
+    const double got = __shfl_sync(all, s, 8 * (rank & 3));
+    if (bad && rank >> 2 == round) keep = got;
+  }
+  return keep;
 }
 
 // T1 = Ahat X (kept in t1, column-major) and its digits by rows
-__global__ void __launch_bounds__(kFarThreads) k_slice_t1(QapTcDev q) {
+__global__ void __launch_bounds__(kFarThreads) k_slice_t1(QapTcDev q, const double* x) {
   tc::pdl_wait();
-  const int r0 = blockIdx.x * 8, i = threadIdx.x & 7, g = threadIdx.x >> 3;
-  if (r0 + i < q.d)
-    for (int k = g; k < q.d; k += 128) q.t1[(size_t)k * q.d + r0 + i] = join(q, 0, kAhat, kXCol, r0 + i, k);
+  const int r0 = blockIdx.x * 8, i = threadIdx.x & 7;
+  const int kw = (threadIdx.x >> 5) * 4, kl = (threadIdx.x & 31) >> 3;   // a warp: eight rows of four columns
+  constexpr int kStep = kFarThreads / 8;
+  for (int c0 = kw; c0 < q.d; c0 += 32 * kStep) {
+    unsigned bad = 0u;   // by step
+    for (int t = 0; t < 32 && c0 + t * kStep < q.d; t++) {
+      const int k = c0 + t * kStep + kl;
+      if (r0 + i >= q.d || k >= q.d) continue;
+      int size;
+      const double v = join(q, 0, kAhat, kXCol, r0 + i, k, size);
+      q.t1[(size_t)k * q.d + r0 + i] = v;
+      if (!reaches(field(v), size) && !(fabs(v) >= least(q, kAhat, kXCol, r0 + i, k) && fabs(v) <= DBL_MAX)) bad |= 1u << t;
+    }
+    unsigned any = __reduce_or_sync(0xffffffffu, bad);
+    for (; any; any &= any - 1u) {
+      const int t = __ffs(any) - 1, k0 = c0 + t * kStep;
+      const bool mine = (bad >> t) & 1u;
+      const double v = dot8(mine, 0.0, q.d, [&](double s, int l, int src) {
+        return fma(q.mats[(size_t)(r0 + (src & 7)) * q.d + l], x[(size_t)(k0 + (src >> 3)) * q.d + l], s);
+      });
+      if (mine) q.t1[(size_t)(k0 + kl) * q.d + r0 + i] = v;
+    }
+  }
   __syncthreads();
   slice_far([&](int r, int k) { return q.t1[(size_t)k * q.d + r]; }, r0, q.d, q.kp, q.plane, q.dig[kT1], q.scale[kT1]);
 }
 
 // out = T1 Bhat - S X - X T
-__global__ void __launch_bounds__(256) k_join(QapTcDev q, double* out) {
+__global__ void __launch_bounds__(256) k_join(QapTcDev q, const double* x, double* out) {
   tc::pdl_wait();
-  const int64_t e = (int64_t)blockIdx.x * 256 + threadIdx.x;
-  if (e >= (int64_t)q.d * q.d) return;
-  const int i = (int)(e % q.d), j = (int)(e / q.d);
-  out[e] = join(q, 3, kT1, kBhat, i, j) - join(q, 1, kS, kXCol, i, j) - join(q, 2, kXRow, kT, i, j);
+  const int64_t e = (int64_t)blockIdx.x * 256 + threadIdx.x, e0 = e - (threadIdx.x & 31), dd = (int64_t)q.d * q.d;
+  const bool in = e < dd;
+  double v = 0.0;
+  bool bad = false;
+  if (in) {
+    const int i = (int)(e % q.d), j = (int)(e / q.d);
+    int sa, sb, sc;
+    const double a = join(q, 3, kT1, kBhat, i, j, sa), b = join(q, 1, kS, kXCol, i, j, sb),
+                 c = join(q, 2, kXRow, kT, i, j, sc);
+    v = a - b - c;
+    if (!reaches(max(field(a), max(field(b), field(c))), max(sa, max(sb, sc)))) {
+      const double most = fabs(a) + fabs(b) + fabs(c);
+      bad = !(most >= least(q, kT1, kBhat, i, j) + least(q, kS, kXCol, i, j) + least(q, kXRow, kT, i, j) && most <= DBL_MAX);
+    }
+  }
+  v = dot8(bad, v, q.d, [&](double s, int t, int src) {
+    const int i = (int)((e0 + src) % q.d);
+    const size_t j = (size_t)((e0 + src) / q.d) * q.d, k = (size_t)t * q.d + i;
+    s = fma(q.t1[k], q.mats[dd + j + t], s);
+    s = fma(-q.mats[2 * dd + (size_t)i * q.d + t], x[j + t], s);
+    return fma(-x[k], q.mats[3 * dd + j + t], s);
+  });
+  if (in) out[e] = v;
 }
 
 struct Maps {
@@ -323,6 +426,7 @@ cudaError_t qap_tc_create(QapTc** out, int64_t d, const double* mats, void* mem,
   QapTc* t = new QapTc();
   QapTcDev& q = t->dev;
   q.d = (int)d;
+  q.mats = mats;
   q.dp = (int)((d + kBM - 1) / kBM * kBM);
   q.kp = (int)((d + kBK - 1) / kBK * kBK);
   q.groups = std::min(q.kp / kBK, kGroups);
@@ -366,10 +470,10 @@ cudaError_t qap_tc_apply(const QapTc* t, const double* x, double* out, bool pdl,
   const dim3 far(kFarThreads), fix(128), flat(256);
   cudaError_t e = tc::launch_kernel(false, 1, k_slice_x, dim3(rows + (q.d + 31) / 32), far, 0, s, x, q);
   if (e == cudaSuccess) e = tc::launch_kernel(pdl, 1, k_fix, dim3(3 * tiles * q.groups), fix, kFixSmem, s, t->one, q, 0);
-  if (e == cudaSuccess) e = tc::launch_kernel(pdl, 1, k_slice_t1, dim3(rows), far, 0, s, q);
+  if (e == cudaSuccess) e = tc::launch_kernel(pdl, 1, k_slice_t1, dim3(rows), far, 0, s, q, x);
   if (e == cudaSuccess) e = tc::launch_kernel(pdl, 1, k_fix, dim3(tiles * q.groups), fix, kFixSmem, s, t->two, q, 3);
   if (e == cudaSuccess)
-    e = tc::launch_kernel(pdl, 1, k_join, dim3((unsigned)(((int64_t)q.d * q.d + 255) / 256)), flat, 0, s, q, out);
+    e = tc::launch_kernel(pdl, 1, k_join, dim3((unsigned)(((int64_t)q.d * q.d + 255) / 256)), flat, 0, s, q, x, out);
   return e;
 }
 

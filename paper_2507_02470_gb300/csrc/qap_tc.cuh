@@ -12,6 +12,7 @@ struct QapTcDev {
   int d, dp, kp;              // size; rows of a digit plane (a multiple of 128), columns (of 64)
   int groups;                 // partial sums per product: chunks of 64 k's are dealt to them in turn
   size_t plane;               // pairs of digits per plane
+  const double* mats;         // Ahat, Bhat, S, T
   uint32_t* dig[kTcMats];     // seven planes each, most significant first
   double* scale[kTcMats];     // 2^(exponent - 34) of every row
   long long* part;            // [product][group][high, low][column][row]
@@ -22,7 +23,7 @@ struct QapTcDev {
 struct QapTc;
 // device memory that a handle provides for size d; part: its pieces
 size_t qap_tc_bytes(int64_t d, size_t (&part)[5]);
-// mats: Ahat, Bhat, S, T on the device (read here only); mem: qap_tc_bytes(d) bytes, 1024-byte aligned
+// mats: Ahat, Bhat, S, T on the device (read by every product); mem: qap_tc_bytes(d) bytes, 1024-byte aligned
 cudaError_t qap_tc_create(QapTc** out, int64_t d, const double* mats, void* mem, cudaStream_t s);
 void qap_tc_free(QapTc* t);
 const int* qap_tc_error(const QapTc* t);   // device word
