@@ -186,7 +186,9 @@ typedef struct hprqp_params {
                                 to 1e9 entries); 0: never.  Sums in another order (rounding only) */
   int32_t wait_polls;        /* launch_mode 3 and the resident launches of launch_mode 0: polls of
                                 one grid-barrier wait before the solve gives up with
-                                HPRQP_TIMEOUT; 0 (default): one to a few seconds */
+                                HPRQP_TIMEOUT; also of a wait for operands in the tensor-core QAP
+                                product (a solve or an apply gives up); 0 (default): one to a few
+                                seconds */
   int32_t batch_team;        /* batched solver: 0 (default) threads per instance chosen per bucket
                                 of n (autotune 1: timed on the batch; 0: 512/256/128/64 from the
                                 largest n down); 64, 128, 256 or 512: that block size for all */
@@ -323,8 +325,9 @@ hprqp_status hprqp_power_noalloc(int64_t m, int64_t n, const int32_t* A_rowptr, 
 void hprqp_destroy(hprqp_handle* h);
 
 /* Bookkeeping, with no counterpart in the paper: sets hprqp_params.wait_polls of the handle for
- * later solves (polls of one grid-barrier wait; 0 restores the default).  A solve
- * whose wait gave up returns HPRQP_TIMEOUT; every solve starts from a cleared barrier. */
+ * later solves (polls of one grid-barrier wait, or of one wait of the tensor-core QAP product; 0
+ * restores the default).  A solve (with the QAP product also an apply) whose wait gave up returns
+ * HPRQP_TIMEOUT; every one starts from a cleared barrier and error word. */
 hprqp_status hprqp_set_wait_polls(hprqp_handle* h, int32_t polls);
 
 /* Bookkeeping, with no counterpart in the paper: the device memory the handle holds, by the

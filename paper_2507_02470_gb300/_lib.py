@@ -311,7 +311,8 @@ class Solver:
         self._keep = []
 
     def set_wait_polls(self, polls):
-        """Polls of one grid-barrier wait before a solve (launch_mode 3, resident launches) gives up (0: default)."""
+        """Polls of one bounded wait before a solve (launch_mode 3, resident launches, tensor-core QAP product) gives up
+        (0: default)."""
         self._check(lib().hprqp_set_wait_polls(self.h, int(polls)))
 
     def set_lambda(self, lambda_A, lambda_Q):

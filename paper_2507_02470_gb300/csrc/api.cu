@@ -1680,7 +1680,16 @@ static hprqp_status power_both(hprqp_handle* h, double* lamA, double* lamQ) {
   return HPRQP_OK;
 }
 
-// A bounded wait of the tensor-core QAP kernels that gave up since the handle was created (the caller has
+// Before a solve or an apply: the tensor-core QAP kernels' error word cleared and their wait limit set
+static hprqp_status qap_arm(hprqp_handle* h) {
+  if (!h->qap_tc) return HPRQP_OK;
+  h->hflags[6] = 0;
+  h->hflags[7] = h->prm.wait_polls;
+  CU(h, cudaMemcpyAsync(qap_tc_error(h->qap_tc), &h->hflags[6], 2 * sizeof(int), cudaMemcpyHostToDevice, h->stream));
+  return HPRQP_OK;
+}
+
+// A bounded wait of the tensor-core QAP kernels that gave up since qap_arm (the caller has
 // nothing in flight on the stream, or waits for it here)
 static hprqp_status qap_check(hprqp_handle* h) {
   if (!h->qap_tc) return HPRQP_OK;
@@ -2062,6 +2071,7 @@ extern "C" hprqp_status hprqp_solve(hprqp_handle* h, double tol, int64_t max_ite
   h->fixed_steps = 0;
   // ---- lambda_A >= lambda_1(AA^*), lambda_Q >= lambda_1(Q) (Sec. 4.1)
   double lamA = 0.0, lamQ = 0.0;
+  if ((st = qap_arm(h))) return st;
   if (h->res.B) {
     const int need = (HA && !(h->prm.lambda_A > 0) ? 1 : 0) | (HQ && !(h->prm.lambda_Q > 0) ? 2 : 0);
     if (need && (st = resident_power(h, need, &lamA, &lamQ))) return st;
@@ -2338,6 +2348,7 @@ extern "C" hprqp_status hprqp_apply(hprqp_handle* h, int32_t op, const double* i
   // with preconditioning the stored operators are E A D, D A^T E, D Q D: map the input into
   // the scaled variables and the output back (A x = E^{-1} A_s D^{-1} x, and so on)
   if (h->scaled) CU(h, launch_vmul((double*)V.ain, op == 1 ? V.ise : V.isd, nin, h->stream));
+  if (const hprqp_status st = qap_arm(h)) return st;
   CU(h, launch_apply(h->args, h->plan, op, h->stream));
   if (h->scaled) CU(h, launch_vmul(V.aout, op == 0 ? V.ise : V.isd, nout, h->stream));
   CU(h, cudaMemcpyAsync(out, V.aout, nout * sizeof(double), cudaMemcpyDefault, h->stream));

@@ -333,8 +333,10 @@ __global__ void __launch_bounds__(128, 1) k_fix(const __grid_constant__ Maps map
       }
     }
     if (threadIdx.x == 32) {
-      // a wait that gives up has recorded its error; a second one lets the copies in flight end
-      if (tc::mbar_wait(full, ph, q.err, 1) || tc::mbar_wait(full, ph, q.err, 1)) {
+      // a wait that gives up has recorded its error; a second one lets the copies in flight end (read from memory: the
+      // launches of a captured graph keep their arguments)
+      const uint32_t polls = (uint32_t)__ldcg(q.err + 1);
+      if (tc::mbar_wait(full, ph, q.err, 1, polls ? polls : tc::kSpin) || tc::mbar_wait(full, ph, q.err, 1)) {
         tc::tc_fence_after();
         constexpr uint32_t idesc = tc::idesc_bf16(kBM, kBN);
         for (int s = 0; s < kSum; s++) {
@@ -402,7 +404,7 @@ struct QapTc {
 };
 
 void qap_tc_free(QapTc* t) { delete t; }
-const int* qap_tc_error(const QapTc* t) { return t->dev.err; }
+int* qap_tc_error(const QapTc* t) { return t->dev.err; }
 
 size_t qap_tc_bytes(int64_t d, size_t (&part)[5]) {
   const int64_t dp = (d + kBM - 1) / kBM * kBM, kp = (d + kBK - 1) / kBK * kBK;

@@ -17,7 +17,7 @@ struct QapTcDev {
   double* scale[kTcMats];     // 2^(exponent - 34) of every row
   long long* part;            // [product][group][high, low][column][row]
   double* t1;
-  int* err;                   // set by a bounded wait that gave up
+  int* err;                   // [0] set by a bounded wait that gave up; [1] polls of a wait for operands (0: kSpin)
 };
 
 struct QapTc;
@@ -26,7 +26,7 @@ size_t qap_tc_bytes(int64_t d, size_t (&part)[5]);
 // mats: Ahat, Bhat, S, T on the device (read by every product); mem: qap_tc_bytes(d) bytes, 1024-byte aligned
 cudaError_t qap_tc_create(QapTc** out, int64_t d, const double* mats, void* mem, cudaStream_t s);
 void qap_tc_free(QapTc* t);
-const int* qap_tc_error(const QapTc* t);   // device word
+int* qap_tc_error(const QapTc* t);   // device words: QapTcDev::err
 // out = vec(Ahat X Bhat - S X - X T): five kernels; pdl: the last four as programmatic dependent launches
 cudaError_t qap_tc_apply(const QapTc* t, const double* x, double* out, bool pdl, cudaStream_t s);
 constexpr int kQapTcKernels = 5;

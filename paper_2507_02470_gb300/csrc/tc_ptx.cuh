@@ -36,9 +36,9 @@ __device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
   return ok != 0;
 }
 
-// waits for that phase; after kSpin polls it gives up and records `code` in *err
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int* err, int code) {
-  for (uint32_t i = 0; i < kSpin; ++i) {
+// waits for that phase; after `polls` polls it gives up and records `code` in *err
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int* err, int code, uint32_t polls = kSpin) {
+  for (uint32_t i = 0; i < polls; ++i) {
     if (mbar_test(bar, parity)) return true;
     if (i >= 64) __nanosleep(200);
   }
