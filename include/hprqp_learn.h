@@ -91,6 +91,10 @@ typedef struct hprqp_mlp hprqp_mlp;
 /* dims: host array of nlayers + 1 widths (each >= 1); max_batch >= 1.  Weights start at 0. */
 hprqp_status hprqp_mlp_create(hprqp_mlp** net, int32_t nlayers, const int32_t* dims, int32_t max_batch,
                               void* stream);
+/* Bookkeeping: the most parts that K is split into in a layer's product (the blocks of one thread-block cluster),
+ * at most 16 and at most what the device holds; 0 restores that largest number, which a new handle
+ * has.  Sums in another order (rounding only). */
+hprqp_status hprqp_mlp_set_cluster(hprqp_mlp* net, int32_t most);
 /* Copies W (dims[l+1] x dims[l], row-major) and b (dims[l+1]) in FP32, host or device, into
  * layer l and clears its Adam moments. */
 hprqp_status hprqp_mlp_set_layer(hprqp_mlp* net, int32_t l, const float* W, const float* b);

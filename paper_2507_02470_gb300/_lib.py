@@ -120,6 +120,7 @@ SIGNATURES = [
     ("hprqp_col_mean_f64", C.c_int, [_vp, _i64, _i64, _i64, _vp, _vp]),
     ("hprqp_ws_standardize", C.c_int, [_vp, _i64, _i64, _i64, _vp, _vp, _vp, _i64, _vp]),
     ("hprqp_mlp_create", C.c_int, [C.POINTER(_vp), _i32, C.POINTER(_i32), _i32, _vp]),
+    ("hprqp_mlp_set_cluster", C.c_int, [_vp, _i32]),
     ("hprqp_mlp_set_layer", C.c_int, [_vp, _i32, _vp, _vp]),
     ("hprqp_mlp_get_layer", C.c_int, [_vp, _i32, _vp, _vp]),
     ("hprqp_mlp_forward", C.c_int, [_vp, _vp, _i64, _i32, _vp, _i64]),

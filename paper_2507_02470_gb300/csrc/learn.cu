@@ -565,6 +565,7 @@ struct hprqp_mlp {
   std::vector<uint16_t*> actB, actT;  // input of layer l: batch-major (maxB x round8(d_l)), feature-major
   std::vector<uint16_t*> dzB, dzT;    // gradient w.r.t. the output of layer l (before ReLU)
   int64_t work_floats = 0;           // bound of the K-splits' partial sums (splits x M x N)
+  int cluster = 1;                   // most K-splits: the blocks of one cluster
   int B = 0;                         // batch of the last forward
   int sms = 148;
   std::vector<void*> allocs;
@@ -600,6 +601,7 @@ extern "C" hprqp_status hprqp_mlp_create(hprqp_mlp** out, int32_t nlayers, const
   n->ldT = round8(max_batch);
   n->s = (cudaStream_t)stream;
   n->sms = device_sms();
+  n->cluster = hprqp::tc::layer_cluster();
   hprqp_status st;
   auto A = [&](void* pp, size_t bytes) { return mlp_alloc(n, reinterpret_cast<void**>(pp), bytes); };
   n->layers.resize(nlayers);
@@ -654,6 +656,14 @@ static LayerSet layer_set(const hprqp_mlp* n, int l0, int l1, F blocks) {
 }
 static int adam_tiles(const MlpLayer& y) { return ((y.din + 31) / 32) * ((y.dout + 31) / 32); }
 
+extern "C" hprqp_status hprqp_mlp_set_cluster(hprqp_mlp* n, int32_t most) {
+  if (!n || most < 0 || most > hprqp::tc::kLayerSplits)
+    return lfail(HPRQP_INVALID_ARG, "mlp_set_cluster: need a handle and 0 <= most <= %d", hprqp::tc::kLayerSplits);
+  const int held = hprqp::tc::layer_cluster();
+  n->cluster = most ? std::min(most, held) : held;
+  return HPRQP_OK;
+}
+
 static hprqp_status refresh_bf16(hprqp_mlp* n, int l) {
   const LayerSet set = layer_set(n, l, l + 1, adam_tiles);
   k_adam<<<set.first[1], dim3(32, 8), 0, n->s>>>(set, 0, 0.f, 0.f, 0.f, 0.f, 1.f, 1.f);
@@ -699,7 +709,7 @@ extern "C" hprqp_status hprqp_mlp_get_grad(hprqp_mlp* n, int32_t l, float* dW, f
 static hprqp_status mlp_gemm(hprqp_mlp* n, int64_t M, int64_t N, int64_t K, const uint16_t* A, int64_t lda,
                              const uint16_t* B, int64_t ldb, const hprqp::tc::Layer& l) {
   // the splits that fill the GPU, at most a cluster's
-  const int sp = std::min(pick_splits(M, N, K, n->work_floats, n->sms), hprqp::tc::kLayerSplits);
+  const int sp = std::min(pick_splits(M, N, K, n->work_floats, n->sms), n->cluster);
   const char* why = nullptr;
   const cudaError_t e = hprqp::tc::gemm_layer(M, N, K, A, lda, B, ldb, sp, l, n->s, &why);
   if (e == cudaErrorInvalidValue && why) return lfail(HPRQP_INVALID_ARG, "gemm: %s", why);

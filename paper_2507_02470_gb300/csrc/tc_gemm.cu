@@ -487,17 +487,25 @@ cudaError_t launch(const CUtensorMap& ta, const CUtensorMap& tb, const Epi& epi,
   return cudaGetLastError();
 }
 
+// Lets the kernel take its shared memory and clusters of 16
+template <int BN, int MODE>
+cudaError_t layer_setup() {
+  static std::once_flag once;
+  static cudaError_t attr = cudaSuccess;
+  std::call_once(once, [] {
+    attr = cudaFuncSetAttribute(k_gemm_layer<BN, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)smem_bytes<BN, EpiStore::kStages>());
+    if (attr == cudaSuccess)
+      attr = cudaFuncSetAttribute(k_gemm_layer<BN, MODE>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  });
+  return attr;
+}
+
 template <int BN, int MODE>
 cudaError_t launch_layer(const CUtensorMap& ta, const CUtensorMap& tb, const EpiLayer& epi, int64_t M, int64_t N,
                          int kb_total, int kb_per, int splits, cudaStream_t s) {
   constexpr uint32_t bytes = smem_bytes<BN, EpiStore::kStages>();
-  static std::once_flag once;
-  static cudaError_t attr = cudaSuccess;
-  std::call_once(once, [] {
-    attr = cudaFuncSetAttribute(k_gemm_layer<BN, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    if (attr == cudaSuccess)
-      attr = cudaFuncSetAttribute(k_gemm_layer<BN, MODE>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  });
+  const cudaError_t attr = layer_setup<BN, MODE>();
   if (attr != cudaSuccess) return attr;
   return launch_kernel(true, splits, k_gemm_layer<BN, MODE>,
                        dim3((unsigned)((M + kBM - 1) / kBM), (unsigned)((N + BN - 1) / BN), (unsigned)splits), dim3(128),
@@ -578,6 +586,29 @@ cudaError_t gemm_decode(int64_t D, int64_t N, int64_t K, const void* A, int64_t 
   if ((e = make_map(&tb, B, N, K, ldb, BN)) != cudaSuccess) return e;
   const EpiDecode epi{alpha, mu, lo, hi, Z, ldz};
   return BN == 64 ? launch<64>(ta, tb, epi, D, N, kb, kb, 1, stream) : launch<128>(ta, tb, epi, D, N, kb, kb, 1, stream);
+}
+
+int layer_cluster() {
+  // asked of the form with the most shared memory and registers; a single block always fits
+  constexpr int BN = 256;
+  const auto k = k_gemm_layer<BN, LAYER_MASK>;
+  int most = 0;
+  cudaLaunchConfig_t cfg = {};
+  cfg.blockDim = dim3(128);
+  cfg.dynamicSmemBytes = smem_bytes<BN, EpiStore::kStages>();
+  cudaLaunchAttribute at[1];
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = at[0].val.clusterDim.y = 1;
+  int c = layer_setup<BN, LAYER_MASK>() == cudaSuccess ? kLayerSplits : 1;
+  for (; c > 1; c /= 2) {
+    at[0].val.clusterDim.z = (unsigned)c;
+    cfg.gridDim = dim3(1, 1, (unsigned)c);
+    if (cudaOccupancyMaxActiveClusters(&most, k, &cfg) == cudaSuccess && most >= 1) break;
+    cudaGetLastError();
+  }
+  return c;
 }
 
 int layer_splits(int64_t K, int splits) {

@@ -47,6 +47,9 @@ struct Layer {
 };
 constexpr int kLayerSplits = 16;              // K-splits of a tile: CTAs of one cluster
 int layer_splits(int64_t K, int splits);      // the splits that a request for `splits` comes to
+// The most K-splits of a layer that the current device can hold as one cluster: kLayerSplits, or the largest power
+// of two below it for which it has a group of that many SMs
+int layer_cluster();
 cudaError_t gemm_layer(int64_t M, int64_t N, int64_t K, const void* A, int64_t lda, const void* B, int64_t ldb,
                        int splits, const Layer& l, cudaStream_t stream, const char** why);
 

@@ -104,6 +104,10 @@ class MLP:
         self.h = h
         self.t = 0
 
+    def set_cluster(self, most):
+        """Most parts that K is split into in a layer's product (0: what the device holds)."""
+        _chk(lib().hprqp_mlp_set_cluster(self.h, int(most)))
+
     def set_layer(self, l, W, b):
         W = np.ascontiguousarray(W, dtype=np.float32)
         b = np.ascontiguousarray(b, dtype=np.float32)
