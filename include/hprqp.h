@@ -61,8 +61,10 @@ typedef enum hprqp_qkind {
                                 then [Ahat X | S | X][Bhat; -X; -T]: on the tensor cores
                                 (autotune 1 and d >= 8; every element within the error bound
                                 of the FP64 sums, d 2^-53 |Ahat| |X| for the first product and
-                                3 d 2^-53 of the magnitudes added for the second), else as
-                                FP64 contractions; at most one such term; not with launch_mode 3 */
+                                3 d 2^-53 of the magnitudes added for the second), else, and
+                                where memory does not hold their operands' digits and sums (354
+                                bytes per entry of X at most), as FP64 contractions; at most one
+                                such term; not with launch_mode 3 */
 } hprqp_qkind;
 
 typedef enum hprqp_phi {
@@ -183,7 +185,7 @@ typedef struct hprqp_params {
                                 factor (sum over B's rows of their squared lengths <= n / 2) is
                                 multiplied in the inner step through the explicit entries of its
                                 B^T B, with no separate pre-pass launch; 2: every such factor (up
-                                to 1e9 entries); 0: never.  Sums in another order (rounding only) */
+                                to 1e9 entries, and where memory holds them); 0: never.  Sums in another order (rounding only) */
   int32_t wait_polls;        /* launch_mode 3 and the resident launches of launch_mode 0: polls of
                                 one grid-barrier wait before the solve gives up with
                                 HPRQP_TIMEOUT; also of a wait for operands in the tensor-core QAP

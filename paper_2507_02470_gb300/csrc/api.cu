@@ -61,6 +61,8 @@ struct hprqp_handle {
   cudaEvent_t pfork = nullptr, pjoin = nullptr;
   // resident solver (resident.cu): its plan (B = 0: not used), barrier flags, partial sums, results
   QapTc* qap_tc = nullptr;   // tensor-core form of the QAP term
+  bool lean = false;         // leave out the forms that take more memory than the problem needs
+  bool extra = false;        // such a form was asked for
   ResPlan res;
   unsigned* res_flags = nullptr;
   double *res_part = nullptr, *res_lam = nullptr;
@@ -1015,7 +1017,7 @@ static hprqp_status create_impl(hprqp_handle* h, int64_t n, int64_t m, const hpr
   QD.tfd = toff;
   if (qap_d) {
     // the QAP product x -> vec(Ahat X Bhat - S X - X T) goes to the intermediate buffers
-    // after the factor rows; cuBLAS runs its four DGEMMs on the handle's stream
+    // after the factor rows
     double *dq, *tmp, *qin;
     if ((st = upload(h, &dq, qap_vals)) || (st = zeros(h, &tmp, (size_t)qap_d * qap_d)) || (st = zeros(h, &qin, n)))
       return st;
@@ -1025,7 +1027,8 @@ static hprqp_status create_impl(hprqp_handle* h, int64_t n, int64_t m, const hpr
     QD.qap_in = qin;
     QD.qap_off = toff;
     toff += n;
-    if (qap_d >= kQapTcMinD && h->prm.autotune == 1) {
+    if (qap_d >= kQapTcMinD && h->prm.autotune == 1 && !h->lean) {
+      h->extra = true;   // up to 354 bytes per entry of X, 96 for digits and 256 for sums
       size_t parts[5];
       void* mem;
       if ((st = dalloc(h, &mem, qap_tc_bytes(qap_d, parts)))) return st;
@@ -1076,7 +1079,10 @@ static hprqp_status create_impl(hprqp_handle* h, int64_t n, int64_t m, const hpr
         const double l = (double)(B.rp[r + 1] - B.rp[r]);
         sq += l * l;
       }
-      if (sq > 0.5 * (double)n && h->prm.factor_inline != 2) continue;
+      if (sq > 0.5 * (double)n) {
+        if (h->prm.factor_inline != 2 || h->lean) continue;
+        h->extra = true;
+      }
       if ((double)pairs + sq > 1e9) continue;
       pairs += (int64_t)sq;
       QD.inl[f] = 1;
@@ -1288,14 +1294,16 @@ static hprqp_status create_impl(hprqp_handle* h, int64_t n, int64_t m, const hpr
   return HPRQP_OK;
 }
 
-extern "C" hprqp_status hprqp_create(hprqp_handle** out, int64_t n, int64_t m, const hprqp_qop* Q,
-                                     const int32_t* A_rowptr, const int32_t* A_colidx, const double* A_vals,
-                                     const double* c, const double* l, const double* u, const double* L,
-                                     const double* U, int32_t phi, double lambda, const hprqp_params* params) {
+// lean: see hprqp_handle; *extra: whether the lean form would take less memory
+static hprqp_status create_handle(hprqp_handle** out, int64_t n, int64_t m, const hprqp_qop* Q,
+                                  const int32_t* A_rowptr, const int32_t* A_colidx, const double* A_vals,
+                                  const double* c, const double* l, const double* u, const double* L, const double* U,
+                                  int32_t phi, double lambda, const hprqp_params* params, bool lean, bool* extra) {
   g_create_err.clear();
   if (!out) return fail(nullptr, HPRQP_INVALID_ARG, "null handle pointer");
   *out = nullptr;
   hprqp_handle* h = new hprqp_handle();
+  h->lean = lean;
   if (params) h->prm = *params;
   else hprqp_default_params(&h->prm);
   if (h->prm.check_every < 1 || h->prm.restart_every < 1 || h->prm.iters_per_launch < 1 ||
@@ -1324,11 +1332,24 @@ extern "C" hprqp_status hprqp_create(hprqp_handle** out, int64_t n, int64_t m, c
   }
   if (st != HPRQP_OK) {
     if (g_create_err.empty()) g_create_err = h->err;
+    *extra = h->extra;
     release(h);
     return st;
   }
   *out = h;
   return HPRQP_OK;
+}
+
+extern "C" hprqp_status hprqp_create(hprqp_handle** out, int64_t n, int64_t m, const hprqp_qop* Q,
+                                     const int32_t* A_rowptr, const int32_t* A_colidx, const double* A_vals,
+                                     const double* c, const double* l, const double* u, const double* L,
+                                     const double* U, int32_t phi, double lambda, const hprqp_params* params) {
+  bool extra = false;
+  const hprqp_status st =
+      create_handle(out, n, m, Q, A_rowptr, A_colidx, A_vals, c, l, u, L, U, phi, lambda, params, false, &extra);
+  if (st != HPRQP_OOM || !extra) return st;
+  // the memory does not hold the digits of a QAP term, or the entries of B^T B that factor_inline = 2 asks for
+  return create_handle(out, n, m, Q, A_rowptr, A_colidx, A_vals, c, l, u, L, U, phi, lambda, params, true, &extra);
 }
 
 // ------------------------------------------------------------------------------------ warm start
