@@ -134,8 +134,8 @@ hprqp_status hprqp_ws_loss(const float* O, int64_t ldo, int32_t B, int32_t r, co
 /* Decoder of the network output O (B x ldo, FP32):
  *   ell[b] = bf16(O[b][1..r]),  sigma0[b] = exp(s_mean + O[b][0] / s_istd),
  *   Z[b][i] = clip(mu[i] + alpha sum_k Phi[i][k] ell[b][k], lo[i], hi[i])   (FP64, i < D)
- * with Phi (D x r, ldphi, BF16).  work: D * B floats (the product now stays on chip: not written).
- * sigma0 may be NULL. */
+ * with Phi (D x r, ldphi, BF16).  work is not used (the product stays on chip) and
+ * may be NULL, like sigma0. */
 hprqp_status hprqp_ws_decode(const uint16_t* Phi, int64_t ldphi, int64_t D, int32_t r, const float* O, int64_t ldo,
                              int32_t B, float alpha, float s_mean, float s_istd, const double* mu, const double* lo,
                              const double* hi, float* work, double* Z, int64_t ldz, double* sigma0, void* stream);

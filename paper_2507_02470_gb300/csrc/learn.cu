@@ -826,11 +826,11 @@ extern "C" hprqp_status hprqp_ws_loss(const float* O, int64_t ldo, int32_t B, in
 
 extern "C" hprqp_status hprqp_ws_decode(const uint16_t* Phi, int64_t ldphi, int64_t D, int32_t r, const float* O,
                                         int64_t ldo, int32_t B, float alpha, float s_mean, float s_istd,
-                                        const double* mu, const double* lo, const double* hi, float* work, double* Z,
+                                        const double* mu, const double* lo, const double* hi, float* /*work*/, double* Z,
                                         int64_t ldz, double* sigma0, void* stream) {
   if (D < 1 || r < 1 || B < 1 || ldo < 1 + r || ldz < D || (B + 31) / 32 > 65535 || (D + 31) / 32 > (int64_t)INT32_MAX)
     return lfail(HPRQP_INVALID_ARG, "ws_decode: bad sizes");
-  if (!Phi || !O || !mu || !lo || !hi || !work || !Z) return lfail(HPRQP_INVALID_ARG, "ws_decode: null pointer");
+  if (!Phi || !O || !mu || !lo || !hi || !Z) return lfail(HPRQP_INVALID_ARG, "ws_decode: null pointer");
   cudaStream_t st = (cudaStream_t)stream;
   const int64_t ldl = round8(r);
   uint16_t* ell = nullptr;

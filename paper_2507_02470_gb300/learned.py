@@ -358,11 +358,10 @@ class LearnedWarmStart:
         for b0 in range(0, B, self.max_batch):
             b1 = min(B, b0 + self.max_batch)
             O = self.mlp.forward(X[b0:b1])
-            work = torch.empty(self.D * (b1 - b0), dtype=torch.float32, device=self.device)
             _chk(lib().hprqp_ws_decode(self.Phi.data_ptr(), self.Phi.stride(0), self.D, self.r, O.data_ptr(),
                                        O.stride(0), b1 - b0, C.c_float(self.alpha), C.c_float(self.s_mean),
                                        C.c_float(self.s_istd), self.mu.data_ptr(), self.lo.data_ptr(),
-                                       self.hi.data_ptr(), work.data_ptr(), Z0[b0:b1].data_ptr(), Z0.stride(0),
+                                       self.hi.data_ptr(), None, Z0[b0:b1].data_ptr(), Z0.stride(0),
                                        sig[b0:b1].data_ptr(), _sp(self.stream)))
         return Z0, sig
 
