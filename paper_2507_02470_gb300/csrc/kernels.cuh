@@ -1058,25 +1058,11 @@ __global__ void __launch_bounds__(kThreads, (VAR == VAR_PLAIN || KIND == K_ATH |
 }
 
 // ------------------------------------------------------------------------------------ restart (Alg. 5)
-__device__ __forceinline__ void sigma_argmin_dev(double t1, double t2, double t3, double lq, int golden,
-                                                 double* out) {
-  double hi = sqrt(t2 / t1);
-  if (t3 <= 0.0 || lq <= 0.0) {
-    *out = hi;
-    return;
-  }
-  double lo = sqrt(t2 / (t1 + t3 / lq));
-  if (!golden) {
-    for (int it = 0; it < 200 && (hi - lo) > 4.0e-16 * hi; it++) {
-      const double mid = 0.5 * (lo + hi);
-      const double d = 1.0 + lq * mid;
-      const double fp = t1 - t2 / (mid * mid) + t3 * mid * (2.0 + lq * mid) / (d * d);
-      if (fp > 0.0) hi = mid;
-      else lo = mid;
-    }
-    *out = 0.5 * (lo + hi);
-    return;
-  }
+// The minimiser of eq. (3.12) by golden-section search on log sigma, by one thread (sigma_golden)
+__device__ __forceinline__ double sigma_argmin_golden(double t1, double t2, double t3, double lq) {
+  const double hi = sqrt(t2 / t1);
+  if (t3 <= 0.0 || lq <= 0.0) return hi;
+  const double lo = sqrt(t2 / (t1 + t3 / lq));
   const double gr = 0.6180339887498949;
   double A = log(lo), B = log(hi);
   double x1 = B - gr * (B - A), x2 = A + gr * (B - A);
@@ -1096,11 +1082,11 @@ __device__ __forceinline__ void sigma_argmin_dev(double t1, double t2, double t3
       f2 = f(x2);
     }
   }
-  *out = exp(0.5 * (A + B));
+  return exp(0.5 * (A + B));
 }
 
 // The exact minimiser of eq. (3.12) by one warp (valid in every lane): the bracket of
-// sigma_argmin_dev, cut into 33 parts per round.  The sign of f' is taken from f' sigma^2
+// sigma_argmin_golden, cut into 33 parts per round.  The sign of f' is taken from f' sigma^2
 // (1 + lQ sigma)^2, which needs no division: a dozen rounds of about ten FP64 operations, where the
 // bisection by one thread took 70 us (50 rounds of three dependent divisions).
 __device__ __forceinline__ double sigma_argmin_warp(double t1, double t2, double t3, double lq) {
@@ -1129,9 +1115,7 @@ __device__ __forceinline__ double sigma_argmin_warp(double t1, double t2, double
 __device__ __forceinline__ void algorithm5(Ctrl& C, double dy2, double wqw, double qwd, double dx2, double th3) {
   const double th1 = fmax(C.lamA * dy2 + C.lamQ * wqw - 2.0 * qwd, 1e-12);
   const double th2 = fmax(dx2, 1e-12);
-  double snew;
-  if (C.sigma_golden) sigma_argmin_dev(th1, th2, th3, C.lamQ, 1, &snew);
-  else snew = sigma_argmin_warp(th1, th2, th3, C.lamQ);
+  const double snew = C.sigma_golden ? sigma_argmin_golden(th1, th2, th3, C.lamQ) : sigma_argmin_warp(th1, th2, th3, C.lamQ);
   const int lane = threadIdx.x & 31;
   const double beta = exp(-C.ratio);
   const double lg = log(lane == 0 ? snew : C.sigma);   // both logarithms at once
