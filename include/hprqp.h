@@ -122,7 +122,9 @@ typedef struct hprqp_params {
   int32_t autotune;          /* 1 (default): time the SpMV schedules (lanes per row 1-32,
                                 the staged form that streams a chunk's entries as one range,
                                 or for A and A^T a SELL-32 copy) at create and pick the
-                                fastest for each operator;
+                                fastest for each operator (a problem that is solved by resident
+                                launches, see launch_mode, is not timed: its separate kernels, for
+                                hprqp_apply and hprqp_profile, take lanes as with 0);
                                 0: lanes per row from the mean row length; 2: the staged
                                 form for every CSR pass; 3: the SELL-32 copy for the A and
                                 A^T passes (rows sorted by length inside each 256-row chunk,
